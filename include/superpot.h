@@ -82,15 +82,21 @@ typedef void* sp_stream; /* a cudaStream_t */
  *   prec       : sp_precision of rho/u and of the solve passes.
  *   max_batch  : largest batch sp_solve_batched will be given (>= 1); the workspace
  *                is sized for it.
- * Device memory: multiplier octant (n0+1)(n1+1)(n2+1) FP64 (+ an FP32 or double-float
- * copy for those passes), twiddles, and a workspace of n0 * 2n1 * (n2+1) complex values
- * per batch element (see sp_plan_workspace_bytes).  Allocated on the current device,
- * stream-ordered from its default memory pool (cudaMallocAsync on a stream of the plan's
- * own, complete when this call returns); sp_plan_create_ex takes a caller's allocator.
- * Every precision takes the same lengths: register-resident passes where every padded
- * length has a compiled plan (2n in {64, 128, 192, 256, 384, 512, 1024}), shared-memory
- * passes (radix 2..8, 3, 5 and 7 stages, or Bluestein's algorithm) elsewhere.  Bluestein
- * axes also hold a table of 2n + 3M complex values built on the host and copied here.
+ * Device memory: multiplier octant (n0+1)(n1+1)(n2+1) FP64, the octant of the passes'
+ * transform lengths F in the pass type, twiddles, and a workspace of n0 * F1 * (F2/2+1)
+ * complex values per batch element (see sp_plan_workspace_bytes).  Allocated on the
+ * current device, stream-ordered from its default memory pool (cudaMallocAsync on a stream
+ * of the plan's own, complete when this call returns); sp_plan_create_ex takes a caller's
+ * allocator.
+ * Every precision takes the same lengths.  Where every 2n has a tuned plan (64, 128, 192,
+ * 256, 384, 512, 1024), F = 2n.  On other grids the solve passes run on the shortest
+ * lengths F >= 2n they are compiled for (4 to 29 % longer in the mean and at most, from 64
+ * up): the same aperiodic convolution, its multiplier carried to period F at precompute, so
+ * the results differ from the 2n transforms by rounding only.  The 2n transforms themselves
+ * (radix 2..8, 3, 5 and 7 stages, or Bluestein's algorithm) serve sp_forward_spectrum, flat
+ * grids whose short axes would round up too far, and a plan whose larger workspace does not
+ * fit the device.  Bluestein axes also hold a table of 2n + 3M complex values built on the
+ * host and copied here.
  */
 sp_status sp_plan_create(sp_plan* out, const int n[3], const double box_lo[3],
                          const double box_hi[3], int padding, const double* gs_w,
@@ -384,7 +390,8 @@ sp_status sp_graph_destroy(sp_graph graph);
  * library (one per GPU that loads the library, held until the process exits) instead
  * of the plan's workspace.  A grid whose workspace, (16 bytes for SP_FP64 and SP_DF32,
  * else 8) x
- * n0 x 2n1 x round_up(n2 + 1, 8), exceeds it is rejected with SP_ERR_UNSUPPORTED_SIZE
+ * n0 x F1 x round_up(F2/2 + 1, 8) (F: the passes' transform lengths, sp_plan_create; the
+ * 2n passes run where only theirs fits), exceeds it is rejected with SP_ERR_UNSUPPORTED_SIZE
  * (of the supported cube sizes, FP64 fits up to n = 126, double-float up to n = 96, its
  * largest supported length below that, and FP32/mixed up to n = 150).
  * The first call on a device looks up the array's device address (once per device,

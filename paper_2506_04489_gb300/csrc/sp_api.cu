@@ -102,10 +102,66 @@ extern "C" sp_status sp_plan_create(sp_plan* out, const int n[3], const double b
     return sp_plan_create_ex(out, n, box_lo, box_hi, padding, gs_w, gs_a, gs_terms, eps, prec, max_batch, nullptr);
 }
 
+int sp_f_length(int N)
+{
+#define SP_F_AT_LEAST(L) \
+    if (N <= L) return L;
+    SP_F_LENGTHS(SP_F_AT_LEAST)
+#undef SP_F_AT_LEAST
+    return 0;
+}
+
+// A grid takes the lengths F unless every padded length has its tuned plan, or the padding to
+// F costs more than the register engine gains over the runtime-radix passes.  That matters
+// only for flat grids, whose short axes round up by up to 8 times.  Gains at equal work:
+// about 2 in FP64 (pipe-bound in both), 2.5 in double-float, 4 and more in FP32, four times
+// that where an axis needs Bluestein's algorithm (512x512x3, growth 2.7: FP64 0.53, double-
+// float 0.96, FP32 1.73 times the speed; 129^3: 11, 12 and 18 times).  Grids of up to 32^3
+// points are bound by latency and gain at any growth measured (7x9x5, growth 3.3: 1.3-1.6).
+bool sp_embeds(const int N[3], sp_precision prec, int F[3])
+{
+    bool tuned = true, blue = false;
+    double growth = 1.0;
+    for (int ax = 0; ax < 3; ++ax) {
+        const bool own = sp_v2_supported(N[ax]);
+        F[ax] = own ? N[ax] : sp_f_length(N[ax]);
+        if (!F[ax]) return false;
+        RadixPlan rp;
+        tuned = tuned && own;
+        blue = blue || !sp_radix_plan(N[ax], &rp);
+        growth *= (double)F[ax] / N[ax];
+    }
+    const bool small = (long long)N[0] * N[1] * N[2] <= 8LL * 32 * 32 * 32;
+    double limit = prec == SP_FP64 ? 1.8 : (prec == SP_DF32 ? 2.5 : 4.0);
+    if (blue) limit *= 4.0;
+    else if (small) limit = 4.0;
+    return !tuned && growth <= limit;
+}
+
+static sp_status create_plan(sp_plan* out, const int n[3], const double box_lo[3],
+                             const double box_hi[3], int padding, const double* gs_w,
+                             const double* gs_a, int gs_terms, double eps,
+                             sp_precision prec, int max_batch, const sp_allocator* allocator, bool may_embed);
+
 extern "C" sp_status sp_plan_create_ex(sp_plan* out, const int n[3], const double box_lo[3],
                                        const double box_hi[3], int padding, const double* gs_w,
                                        const double* gs_a, int gs_terms, double eps,
                                        sp_precision prec, int max_batch, const sp_allocator* allocator)
+{
+    const sp_status rc = create_plan(out, n, box_lo, box_hi, padding, gs_w, gs_a, gs_terms, eps, prec, max_batch,
+                                     allocator, true);
+    // the longer transforms need a larger workspace: without the memory, the 2n passes
+    if (rc != SP_ERR_OOM) return rc;
+    int N[3], F[3];
+    for (int ax = 0; ax < 3; ++ax) N[ax] = 2 * n[ax];
+    if (!sp_embeds(N, prec, F)) return rc;
+    return create_plan(out, n, box_lo, box_hi, padding, gs_w, gs_a, gs_terms, eps, prec, max_batch, allocator, false);
+}
+
+static sp_status create_plan(sp_plan* out, const int n[3], const double box_lo[3],
+                             const double box_hi[3], int padding, const double* gs_w,
+                             const double* gs_a, int gs_terms, double eps,
+                             sp_precision prec, int max_batch, const sp_allocator* allocator, bool may_embed)
 {
     g_err[0] = 0;
     if (!out) return sp_fail(SP_ERR_INVALID, "out is NULL");
@@ -162,6 +218,13 @@ extern "C" sp_status sp_plan_create_ex(sp_plan* out, const int n[3], const doubl
     p->max_batch = max_batch;
     p->ldz = (n[2] + 1 + 7) & ~7;
     p->plane = 2LL * n[1] * p->ldz;
+    const size_t csize = (prec == SP_FP64 || prec == SP_DF32) ? 16 : 8;
+    p->emb = sp_embeds(p->N, prec, p->F) && may_embed;
+    if (!p->emb)
+        for (int ax = 0; ax < 3; ++ax) p->F[ax] = p->N[ax];
+    p->ldf = (p->F[2] / 2 + 1 + 7) & ~7;
+    p->planef = (long long)p->F[1] * p->ldf;
+    p->keep_n = p->emb && csize * n[0] * p->plane <= SP_NOALLOC_MAX_BYTES && csize * n[0] * p->planef > SP_NOALLOC_MAX_BYTES;
     p->eps = eps;
     p->delta = sqrt(p->L[0] * p->L[0] + p->L[1] * p->L[1] + p->L[2] * p->L[2]);
     p->h_tau = 0.1;
@@ -222,8 +285,15 @@ extern "C" sp_status sp_plan_create_ex(sp_plan* out, const int n[3], const doubl
     }
     const size_t mcount = (size_t)(n[0] + 1) * (n[1] + 1) * p->ldz;
     SP_ALLOC(p->d_M64, sizeof(double) * mcount);
-    if (prec == SP_FP32 || prec == SP_MIXED) SP_ALLOC(p->d_M32, sizeof(float) * mcount);
-    if (prec == SP_DF32) SP_ALLOC(p->d_Mdf, sizeof(df32) * mcount);
+    if (!p->emb || p->keep_n) {
+        if (prec == SP_FP32 || prec == SP_MIXED) SP_ALLOC(p->d_M32, sizeof(float) * mcount);
+        if (prec == SP_DF32) SP_ALLOC(p->d_Mdf, sizeof(df32) * mcount);
+    }
+    if (p->emb) {
+        SP_ALLOC(p->d_Ms, csize / 2 * (size_t)(p->F[0] / 2 + 1) * (p->F[1] / 2 + 1) * p->ldf);
+        for (int ax = 0; ax < 3; ++ax)
+            if (!sp_v2_supported(p->N[ax])) SP_ALLOC(p->d_twF[ax], csize * (p->F[ax] + SP_TW_STAGED_MAX));
+    }
     for (int ax = 0; ax < 3; ++ax) {
         SP_ALLOC(p->d_tw64[ax], sizeof(cpx<double>) * p->N[ax]);
         SP_ALLOC(p->d_tw32[ax], sizeof(cpx<float>) * (p->N[ax] + SP_TW_STAGED_MAX));
@@ -243,8 +313,7 @@ extern "C" sp_status sp_plan_create_ex(sp_plan* out, const int n[3], const doubl
             return rc;
         }
     }
-    const size_t csize = (prec == SP_FP64 || prec == SP_DF32) ? 16 : 8;
-    p->work_bytes = csize * (size_t)max_batch * n[0] * (size_t)p->plane;
+    p->work_bytes = csize * (size_t)max_batch * n[0] * (size_t)p->planef;
     SP_ALLOC(p->d_work, p->work_bytes);
 #undef SP_ALLOC
     const cudaError_t ce = p->mem_st ? cudaMemsetAsync(p->d_status, 0, 256, p->mem_st) : cudaMemset(p->d_status, 0, 256);

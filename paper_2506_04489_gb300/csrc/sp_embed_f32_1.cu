@@ -1,0 +1,4 @@
+// FP32 (and mixed) passes of sp_embed.cuh, length group 1, compiled apart to keep translation units small.
+#include "sp_embed.cuh"
+
+SP_F_GROUP1(SP_EMBED_FLOAT, )

@@ -1,0 +1,4 @@
+// native FP64 passes of sp_embed.cuh, length group 2, compiled apart to keep translation units small.
+#include "sp_embed.cuh"
+
+SP_F_GROUP2(SP_EMBED_DOUBLE, )

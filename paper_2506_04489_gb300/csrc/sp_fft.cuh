@@ -41,6 +41,25 @@ template <> SP_D cpx<df32> tw_mulc<df32>(cpx<df32> a, cpx<df32> w)
     const df32 ar = re_of(a), ai = im_of(a), wr = re_of(w), wi = im_of(w);
     return mk(df_dot_add(ar, wr, ai, wi), df_dot_sub(ai, wr, ar, wi));
 }
+// a times an exact power of two; a s + b t with real s, t; -a
+template <class R> SP_D cpx<R> scale_exact(cpx<R> a, float p) { return scale(a, (R)p); }
+template <> SP_D cpx<df32> scale_exact<df32>(cpx<df32> a, float p)
+{
+    a.rh = __fmul_rn(a.rh, p);
+    a.ih = __fmul_rn(a.ih, p);
+    a.rl = __fmul_rn(a.rl, p);
+    a.il = __fmul_rn(a.il, p);
+    return a;
+}
+template <class R> SP_D cpx<R> dot2(cpx<R> a, R s, cpx<R> b, R t)
+{
+    return mk(a.re * s + b.re * t, a.im * s + b.im * t);
+}
+template <> SP_D cpx<df32> dot2<df32>(cpx<df32> a, df32 s, cpx<df32> b, df32 t)
+{
+    return mk(df_dot_add(re_of(a), s, re_of(b), t), df_dot_add(im_of(a), s, im_of(b), t));
+}
+template <class R> SP_D cpx<R> neg(cpx<R> a) { return mk(-re_of(a), -im_of(a)); }
 // Values written to global memory are renormalised.  Exchanges through shared memory
 // between the stages of one transform keep the pair as the arithmetic left it: sums and
 // products accept a low part of a few ulps of the high part (their error stays a small
@@ -49,6 +68,14 @@ template <class R> SP_D cpx<R> norm(cpx<R> a) { return a; }
 template <> SP_D cpx<df32> norm<df32>(cpx<df32> a) { return df_norm_c(a); }
 
 // ------------------------------------------------------------------ plans
+template <int... Rs> struct Radices {
+    static constexpr int NS = sizeof...(Rs);
+    static constexpr int R[sizeof...(Rs)] = {Rs...};
+};
+// E values a thread, forward radices in order
+template <int E_, int... Rs> struct PlanE : Radices<Rs...> {
+    static constexpr int E = E_;
+};
 // Forward radices: powers of two first (the first stage is radix 8 or 16, so zero padding
 // prunes it uniformly), then 3s.  E is a multiple of every radix.
 template <int N> struct FFTPlan;
@@ -99,6 +126,41 @@ struct Plan1024Radix32 {
 template <> struct PlanOf<float, 1024> : Plan1024Radix32 {};
 template <> struct PlanOf<double, 1024> : Plan1024Radix16 {};
 template <> struct PlanOf<df32, 384> : Plan384Radix4 {};
+// Lengths of the passes on grids whose own padded length has no plan above (sp_embed.cuh).
+// First radices of 4, 6, 8, 10, 12, 16 or 20 points, so that the zero half is pruned; the
+// radices 6 to 20 are prime-factor products without inner twiddles.  Plans were chosen by
+// timing the x pass of an n^3 grid with every order of such radices, E values a thread and
+// register caps: 16-byte values want 8 to 12 values a thread (double-float at 200: 82 us
+// with 10-10-2 and E = 10, 104 us with 20-10 and E = 20), FP32 wants fewer stages (at 400:
+// 20-20 and E = 20, 4.6 ps a point, against 5.8 with 10-10-4).
+template <> struct FFTPlan<16> : PlanE<4, 4, 4> {};
+template <> struct FFTPlan<32> : PlanE<8, 8, 4> {};
+template <> struct FFTPlan<48> : PlanE<12, 12, 4> {};
+template <> struct FFTPlan<72> : PlanE<12, 12, 6> {};
+template <> struct FFTPlan<80> : PlanE<20, 20, 4> {};
+template <> struct FFTPlan<96> : PlanE<12, 6, 4, 4> {};
+template <> struct FFTPlan<144> : PlanE<12, 12, 12> {};
+template <> struct FFTPlan<160> : PlanE<20, 20, 4, 2> {};
+template <> struct FFTPlan<200> : PlanE<10, 10, 10, 2> {};
+template <> struct FFTPlan<216> : PlanE<6, 6, 6, 6> {};
+template <> struct FFTPlan<288> : PlanE<12, 12, 6, 4> {};
+template <> struct FFTPlan<320> : PlanE<20, 20, 4, 4> {};
+template <> struct FFTPlan<400> : PlanE<10, 10, 10, 2, 2> {};
+template <> struct FFTPlan<432> : PlanE<12, 12, 6, 6> {};
+template <> struct FFTPlan<576> : PlanE<12, 12, 12, 4> {};
+template <> struct FFTPlan<640> : PlanE<20, 20, 2, 4, 4> {};
+template <> struct FFTPlan<768> : PlanE<12, 4, 4, 4, 12> {};
+template <> struct FFTPlan<864> : PlanE<12, 12, 12, 6> {};
+template <> struct FFTPlan<1280> : PlanE<20, 20, 4, 4, 4> {};
+template <> struct FFTPlan<1536> : PlanE<12, 12, 4, 4, 4, 2> {};
+template <> struct FFTPlan<2048> : PlanE<16, 16, 16, 8> {};
+template <> struct PlanOf<float, 96> : PlanE<24, 12, 8> {};
+template <> struct PlanOf<float, 160> : PlanE<20, 10, 4, 4> {};
+template <> struct PlanOf<float, 200> : PlanE<20, 20, 10> {};
+template <> struct PlanOf<float, 400> : PlanE<20, 20, 20> {};
+template <> struct PlanOf<float, 640> : PlanE<20, 4, 4, 4, 10> {};
+template <> struct PlanOf<float, 768> : PlanE<24, 8, 8, 12> {};
+
 // Plan key of the z passes (contiguous real lines, packed in pairs): the type's own plan,
 // except FP32 at 512 and 1024, whose z passes run faster on 8-8-8 and 16-8-8 than on the
 // radix-32 plans of its line passes.  Each axis has its own staged twiddle table, so the
@@ -309,9 +371,131 @@ template <int S, class R> SP_D void bf32_half(cpx<R>* u)
     bf32_tail<S>(u, e, o);
 }
 
+// radix 4 with u[2] = u[3] = 0
+template <int S, class R> SP_D void bf4_half(cpx<R>* u)
+{
+    const cpx<R> a = u[0], b = u[1], d = mul_si<S>(u[1]);
+    u[0] = a + b;
+    u[1] = a + d;
+    u[2] = a - b;
+    u[3] = a - d;
+}
+
+// radix 5: with t1 = u1 + u4, t2 = u2 + u3, v1 = u1 - u4, v2 = u2 - u3 and s = t1 + t2,
+// the cosine sums are (u0 - s/4) +- (t1 - t2) sqrt(5)/4 (cos(2 pi/5) + cos(4 pi/5) = -1/2,
+// their difference sqrt(5)/2): one real product instead of four.
+template <int S, class R> SP_D void bf5(cpx<R>* u)
+{
+    const R s5 = Num<R>::c(0.559016994374947424102293417182819059);  // sqrt(5)/4
+    const R s1 = Num<R>::c(0.951056516295153572116439333379382143);  // sin(2 pi/5)
+    const R s2 = Num<R>::c(0.587785252292473129168705954639072769);  // sin(4 pi/5)
+    const cpx<R> t1 = u[1] + u[4], t2 = u[2] + u[3], v1 = u[1] - u[4], v2 = u[2] - u[3];
+    const cpx<R> s = t1 + t2, d = scale(t1 - t2, s5);
+    const cpx<R> m = u[0] - scale_exact(s, 0.25f);
+    const cpx<R> a1 = m + d, a2 = m - d;
+    const cpx<R> b1 = mul_si<S>(dot2(v1, s1, v2, s2)), b2 = mul_si<S>(dot2(v1, s2, v2, -s1));
+    u[0] = u[0] + s;
+    u[1] = a1 + b1;
+    u[4] = a1 - b1;
+    u[2] = a2 + b2;
+    u[3] = a2 - b2;
+}
+
+// a times (S i)^m, m mod 4 known at compile time
+template <int S, int M, class R> SP_D cpx<R> rot4(cpx<R> a)
+{
+    if constexpr ((M & 3) == 0) return a;
+    else if constexpr ((M & 3) == 1) return mul_si<S>(a);
+    else if constexpr ((M & 3) == 2) return neg(a);
+    else return mul_si<-S>(a);
+}
+
+// DFT of length A = 2 or 4 of which only the half of the inputs starting at cyclic
+// position P is nonzero: w[P] (A = 2), w[P] and w[P + 1 mod 4] (A = 4).
+template <int S, int A, int P, class R> SP_D void bf_half_at(cpx<R>* w)
+{
+    if constexpr (A == 2) {
+        const cpx<R> a = w[P];
+        w[0] = a;
+        w[1] = P ? neg(a) : a;
+    } else {
+        // sum over d = 0, 1 of w[P + d] (S i)^{(P + d) k}
+        const cpx<R> a = w[P], b = w[(P + 1) & 3], d = mul_si<S>(b);
+        w[0] = a + b;
+        w[1] = rot4<S, P>(a + d);
+        w[2] = rot4<S, 2 * P>(a - b);
+        w[3] = rot4<S, 3 * P>(a - d);
+    }
+}
+
+// Radix A B with A and B coprime (A = 2 or 4, B = 3 or 5) by the prime-factor map: input
+// j = B j1 + A j2 mod A B, output q = B (B^-1 mod A) k1 + A (A^-1 mod B) k2 mod A B, B
+// transforms of length A and A of length B with no twiddles between them.  With the upper
+// half of the inputs zero (HALF) each length-A transform has A/2 cyclically adjacent
+// nonzero inputs.
+template <int A, int B> struct Pfa {
+    static constexpr int N = A * B;
+    static constexpr int inv(int a, int m)
+    {
+        for (int x = 1; x < m; ++x)
+            if (a * x % m == 1) return x;
+        return 1;
+    }
+    static constexpr int in(int j1, int j2) { return (B * j1 + A * j2) % N; }
+    static constexpr int out(int k1, int k2) { return (B * inv(B % A, A) * k1 + A * inv(A % B, B) * k2) % N; }
+    // first of the cyclically adjacent j1 whose input lies in the lower half
+    static constexpr int first(int j2)
+    {
+        for (int j1 = 0; j1 < A; ++j1)
+            if (in(j1, j2) < N / 2 && (A == 2 || in((j1 + A - 1) % A, j2) >= N / 2)) return j1;
+        return 0;
+    }
+};
+template <int S, int A, int B, bool HALF, int J2 = 0, class R> SP_D void pfa_rows(cpx<R>* u, cpx<R> (*w)[A])
+{
+    if constexpr (J2 < B) {
+        using F = Pfa<A, B>;
+#pragma unroll
+        for (int j1 = 0; j1 < A; ++j1) w[J2][j1] = u[F::in(j1, J2)];
+        if constexpr (HALF) bf_half_at<S, A, F::first(J2)>(w[J2]);
+        else if constexpr (A == 4) bf4<S>(w[J2]);
+        else bf2<S>(w[J2]);
+        pfa_rows<S, A, B, HALF, J2 + 1>(u, w);
+    }
+}
+template <int S, int A, int B, bool HALF, class R> SP_D void bf_pfa(cpx<R>* u)
+{
+    using F = Pfa<A, B>;
+    cpx<R> w[B][A];
+    pfa_rows<S, A, B, HALF>(u, w);
+#pragma unroll
+    for (int k1 = 0; k1 < A; ++k1) {
+        cpx<R> x[B];
+#pragma unroll
+        for (int j2 = 0; j2 < B; ++j2) x[j2] = w[j2][k1];
+        if constexpr (B == 3) bf3<S>(x);
+        else bf5<S>(x);
+#pragma unroll
+        for (int k2 = 0; k2 < B; ++k2) u[F::out(k1, k2)] = x[k2];
+    }
+}
+
 template <int RAD, int S, bool HALF, class R> SP_D void butterfly(cpx<R>* u)
 {
-    if constexpr (RAD == 32) {
+    if constexpr (RAD == 20) {
+        bf_pfa<S, 4, 5, HALF>(u);
+    } else if constexpr (RAD == 12) {
+        bf_pfa<S, 4, 3, HALF>(u);
+    } else if constexpr (RAD == 10) {
+        bf_pfa<S, 2, 5, HALF>(u);
+    } else if constexpr (RAD == 6) {
+        bf_pfa<S, 2, 3, HALF>(u);
+    } else if constexpr (RAD == 5) {
+        static_assert(!HALF, "an odd radix cannot run first: its zero inputs are not half");
+        bf5<S>(u);
+    } else if constexpr (RAD == 4 && HALF) {
+        bf4_half<S>(u);
+    } else if constexpr (RAD == 32) {
         if constexpr (HALF) bf32_half<S>(u);
         else bf32<S>(u);
     } else if constexpr (RAD == 16) {
@@ -370,15 +554,14 @@ SP_D void fill_stage_twiddles(cpx<R>* tws, const cpx<R>* __restrict__ tw, int ti
     }
 }
 
-// A plan is usable when its radices multiply to N, every radix divides E (each thread
-// runs whole butterflies) and every stage stride N / radix is a multiple of 8 (the
-// layouts' step rule).
+// A plan is usable when its radices multiply to N and every radix divides E (each thread
+// runs whole butterflies).
 template <class K, int N> constexpr bool plan_ok()
 {
     int prod = 1;
     for (int i = 0; i < PlanOf<K, N>::NS; ++i) {
         const int r = PlanOf<K, N>::R[i];
-        if (PlanOf<K, N>::E % r != 0 || (N / r) % 8 != 0) return false;
+        if (PlanOf<K, N>::E % r != 0) return false;
         prod *= r;
     }
     return prod == N;
@@ -391,17 +574,22 @@ template <class R, int N, bool INV, int ST, class K = R> struct Stage {
     static constexpr int RAD = radix_at<K, N, INV>(ST);
     static constexpr int P = span_at<K, N, INV>(ST);
     static constexpr int NB = E / RAD;
-    static constexpr int STRIDE = N / RAD;  // a multiple of 8 for every plan
+    static constexpr int STRIDE = N / RAD;
 
     // inputs of this stage from shared memory: v[m RAD + r] = x[t + T m + r N/RAD]
     template <class Lay> SP_D static void load(cpx<R> (&v)[E], const cpx<R>* sm, const Lay& lay, int t)
     {
 #pragma unroll
         for (int m = 0; m < NB; ++m) {
-            const cpx<R>* p0 = sm + lay(t + T * m);
-            const int st = lay.step(STRIDE);
+            if constexpr (STRIDE % 8 == 0) {
+                const cpx<R>* p0 = sm + lay(t + T * m);
+                const int st = lay.step(STRIDE);
 #pragma unroll
-            for (int r = 0; r < RAD; ++r) v[m * RAD + r] = p0[r * st];
+                for (int r = 0; r < RAD; ++r) v[m * RAD + r] = p0[r * st];
+            } else {
+#pragma unroll
+                for (int r = 0; r < RAD; ++r) v[m * RAD + r] = sm[lay(t + T * m + r * STRIDE)];
+            }
         }
     }
 

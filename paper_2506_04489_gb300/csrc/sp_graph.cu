@@ -91,7 +91,16 @@ extern "C" sp_status sp_plan_launch_config(const sp_plan p, int* line_tiles, int
         for (int i = 0; i < 24; ++i) radices[i] = 0;
         bool v2 = true;
         for (int ax = 0; ax < 3; ++ax) v2 = v2 && sp_v2_supported(p->N[ax]);
-        if (v2) {
+        if (p->emb) {
+            sp_status rc = SP_OK;
+            switch (p->prec) {
+                case SP_FP64: rc = sp_embed_radices_f64(p, radices); break;
+                case SP_FP32:
+                case SP_MIXED: rc = sp_embed_radices_f32(p, radices); break;
+                case SP_DF32: rc = sp_embed_radices_df(p, radices); break;
+            }
+            if (rc) return rc;
+        } else if (v2) {
             sp_status rc = SP_OK;
             switch (p->prec) {
                 case SP_FP64: rc = sp_v2_radices_f64(p, radices); break;

@@ -11,9 +11,27 @@
 #include "sp_common.cuh"
 #include "sp_df32.cuh"
 
+// Transform lengths of the solve passes on grids whose own padded length 2n has no tuned
+// plan (sp_embed.cuh), increasing.  Steps between neighbours stay below 1.29 from 64 up.
+#define SP_F_LENGTHS(X)                                                                                \
+    X(16) X(32) X(48) X(64) X(72) X(80) X(96) X(128) X(144) X(160) X(192) X(200) X(216) X(256) X(288)  \
+    X(320) X(384) X(400) X(432) X(512) X(576) X(640) X(768) X(864) X(1024) X(1280) X(1536) X(2048)
+
 struct sp_plan_s {
     int n[3];        // grid points per axis
     int N[3];        // padded FFT lengths 2n
+    // Solve passes on lengths F >= N (sp_embed.cuh) when some axis length N has no tuned
+    // plan: the multiplier of period F in the pass type, [|k1|][|k0|][kz] with row stride
+    // ldf; twiddles of the axes with no tuned plan (F base entries, then the staged tables);
+    // planef complex workspace elements per x-plane.  Without it F = N, ldf = ldz, planef =
+    // plane.  keep_n: the 2n multiplier in the pass type is kept as well (sp_solve_noalloc
+    // runs the 2n passes where only their workspace fits its scratch).
+    bool emb, keep_n;
+    int F[3];
+    int ldf;
+    long long planef;
+    void* d_Ms;
+    void* d_twF[3];
     double lo[3], hi[3];
     double h[3];     // grid spacing (hi - lo)/(n - 1)
     double L[3];     // window half-width n h
@@ -71,8 +89,8 @@ struct sp_plan_s {
     // destroy never waits for the device
     cudaStream_t mem_st;
     int nalloc;
-    void* alloc_ptr[32];
-    size_t alloc_bytes[32];
+    void* alloc_ptr[48];
+    size_t alloc_bytes[48];
     // sp_solve_host staging (created by its first call): two input and two output device
     // buffers, a host-to-device and a device-to-host copy stream, and their events
     void* d_stage[4];
@@ -136,6 +154,19 @@ sp_status sp_v2_forward_f32(sp_plan p, const void* rho, void* spec, cudaStream_t
 sp_status sp_v2_forward_f64(sp_plan p, const void* rho, void* spec, cudaStream_t st);
 sp_status sp_v2_forward_df(sp_plan p, const void* rho, void* spec, cudaStream_t st);
 bool sp_v2_supported(int N);
+// Shortest transform length of the solve passes for a padded length N <= 2048 (N itself
+// where it has a tuned plan), and whether a grid with these padded lengths takes them.
+int sp_f_length(int N);
+bool sp_embeds(const int N[3], sp_precision prec, int F[3]);
+sp_status sp_embed_solve_f32(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st, bool mixed);
+sp_status sp_embed_solve_f64(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st);
+sp_status sp_embed_solve_df(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st);
+sp_status sp_embed_twiddles_f32(sp_plan p, cudaStream_t st);
+sp_status sp_embed_twiddles_f64(sp_plan p, cudaStream_t st);
+sp_status sp_embed_twiddles_df(sp_plan p, cudaStream_t st);
+sp_status sp_embed_radices_f32(sp_plan p, int* out);
+sp_status sp_embed_radices_f64(sp_plan p, int* out);
+sp_status sp_embed_radices_df(sp_plan p, int* out);
 // Double-float and FP32 plans keep, after the N base twiddles of an axis, the per-stage
 // twiddle tables that their passes read from global memory; room for this many entries
 // is reserved.

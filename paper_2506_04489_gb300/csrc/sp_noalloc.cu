@@ -59,7 +59,9 @@ extern "C" sp_status sp_solve_noalloc(const sp_plan p, const void* rho, void* u,
     if (!rho || !u) return sp_fail(SP_ERR_INVALID, "rho and u must be non-NULL device pointers");
     if (!p->ready) return sp_fail(SP_ERR_NOT_READY, "sp_kernel_precompute has not been run on this plan");
     const size_t csize = (p->prec == SP_FP64 || p->prec == SP_DF32) ? 16 : 8;
-    const size_t need = csize * (size_t)p->n[0] * (size_t)p->plane;
+    // where the workspace of the plan's own transform lengths does not fit but that of the
+    // 2n passes does, the 2n passes run (keep_n: the plan holds their multiplier)
+    const size_t need = csize * (size_t)p->n[0] * (size_t)(p->keep_n ? p->plane : p->planef);
     if (need > kScratchBytes)
         return sp_fail(SP_ERR_UNSUPPORTED_SIZE,
                        "sp_solve_noalloc: this grid needs %zu bytes of workspace; the static scratch holds %zu",
@@ -78,6 +80,7 @@ extern "C" sp_status sp_solve_noalloc(const sp_plan p, const void* rho, void* u,
     view.work_bytes = need;
     view.max_batch = 1;
     view.timing = false;
+    if (p->keep_n) view.emb = false;
     if ((rc = sp_run_solve(&view, rho, u, 1, (cudaStream_t)stream))) return rc;
     // the plan's completion event (recording it allocates nothing): sp_plan_destroy
     // waits for it before freeing the multiplier and twiddles this solve reads

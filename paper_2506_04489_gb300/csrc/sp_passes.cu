@@ -456,6 +456,14 @@ sp_status sp_run_solve(sp_plan p, const void* rho, void* u, int batch, cudaStrea
             case SP_DF32: return sp_v2_persistent_df(p, rho, u, batch, st);
         }
     }
+    if (p->emb) {  // register-resident passes on longer transforms (sp_embed.cuh)
+        switch (p->prec) {
+            case SP_FP64: return sp_embed_solve_f64(p, rho, u, batch, st);
+            case SP_FP32: return sp_embed_solve_f32(p, rho, u, batch, st, false);
+            case SP_MIXED: return sp_embed_solve_f32(p, rho, u, batch, st, true);
+            case SP_DF32: return sp_embed_solve_df(p, rho, u, batch, st);
+        }
+    }
     // register-resident passes where every axis length has a compiled plan
     sp_status rc = SP_ERR_UNSUPPORTED_SIZE;
     switch (p->prec) {

@@ -120,8 +120,12 @@ size_t entry_bytes(const Srv* s, int n, sp_precision p)
 {
     const size_t c = (p == SP_FP64 || p == SP_DF32) ? 16 : 8, r = io_size(p);
     const size_t ldz = (size_t)(n + 1 + 7) / 8 * 8, nn = (size_t)n;
-    const size_t work = (size_t)s->cfg.max_batch * c * nn * 2 * nn * ldz;
-    const size_t tables = (nn + 1) * (nn + 1) * ldz * (8 + (p == SP_DF32 ? 8 : 4)) + 3 * 2 * nn * 32;
+    const int N[3] = {2 * n, 2 * n, 2 * n};
+    int F[3];
+    const size_t f = sp_embeds(N, p, F) ? (size_t)F[0] : 2 * nn;  // transform length of the passes
+    const size_t ldf = (f / 2 + 1 + 7) / 8 * 8;
+    const size_t work = (size_t)s->cfg.max_batch * c * nn * f * ldf;
+    const size_t tables = (nn + 1) * (nn + 1) * ldz * 8 + (f / 2 + 1) * (f / 2 + 1) * ldf * (p == SP_DF32 ? 8 : 4) + 3 * 2 * nn * 32;
     const size_t io = 2 * (size_t)s->cfg.max_batch * nn * nn * nn * r;
     return work + tables + io + (1u << 20);
 }

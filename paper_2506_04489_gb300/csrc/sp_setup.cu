@@ -309,9 +309,104 @@ __global__ void k_twiddles(int N, cpx<double>* tw64, cpx<float>* tw32, cpx<df32>
     if (j >= N) return;
     double s, c;
     sincospi(2.0 * (double)j / (double)N, &s, &c);
-    tw64[j] = mk(c, -s);
-    tw32[j] = mk((float)c, (float)-s);
-    twdf[j] = mk(df_from_double(c), df_from_double(-s));
+    if (tw64) tw64[j] = mk(c, -s);
+    if (tw32) tw32[j] = mk((float)c, (float)-s);
+    if (twdf) twdf[j] = mk(df_from_double(c), df_from_double(-s));
+}
+
+// ------------------------------------------------------------------------- period F
+// Rows of the change of period of one axis (sp_embed.cuh): the multiplier of period F from
+// the one of period N = 2n, through the kernel values it stands for,
+//   K_j = sum_{k=0}^{N-1} M_k cos(2 pi jk/N),   M'_q = (1/F) sum_{|j| <= n-1} K_j cos(2 pi jq/F),
+// folded over |k|: T[q][k] = (1/F) c_k sum_{|j| <= n-1} cos(2 pi jk/N) cos(2 pi jq/F), c_0 =
+// c_n = 1, else 2.  The sum is half of D(b) + D(b') with b, b' = 2 pi (q/F -+ k/N) and the
+// Dirichlet kernel D(b) = sin((n - 1/2) b) / sin(b/2) = sum_{|j| <= n-1} cos(jb); with
+// b/2 = pi m / (N F), m = q N -+ k F, both phases are reduced as integers.
+__device__ __forceinline__ double dirichlet(long long m, long long NF, int n)
+{
+    // D has period NF in m (both sines change sign); the phases are folded to at most pi/2, so
+    // that neither sine is taken near a multiple of pi of a rounded argument
+    long long r = m % NF;
+    if (2 * r > NF) r -= NF;
+    if (2 * r < -NF) r += NF;
+    if (r == 0) return (double)(2 * n - 1);
+    long long s = (2 * n - 1) * r % (2 * NF);
+    if (s > NF) s -= 2 * NF;
+    if (s < -NF) s += 2 * NF;
+    if (2 * s > NF) s = NF - s;
+    if (2 * s < -NF) s = -NF - s;
+    return sinpi((double)s / (double)NF) / sinpi((double)r / (double)NF);
+}
+__global__ void k_period_rows(int n, int F, double* T)
+{
+    const int nk = n + 1, nq = F / 2 + 1;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= nk * nq) return;
+    const int q = idx / nk, k = idx % nk;
+    const long long N = 2 * n, NF = N * F;
+    const double d = dirichlet(q * N - (long long)k * F, NF, n) + dirichlet(q * N + (long long)k * F, NF, n);
+    T[idx] = (k == 0 || k == n ? 0.5 : 1.0) * d / (double)F;
+}
+
+// C[b][m][j] = sum_k A[m][k] B[b][k][j]: the change of period along a strided axis (FP64,
+// tiles as in k_dgemm_nt).  B's rows have stride ldb, its batches sb; C's likewise.
+__global__ void __launch_bounds__(256) k_dgemm_nn(int M, int N, int K, const double* __restrict__ A,
+                                                  const double* __restrict__ B, long long ldb, long long sb,
+                                                  double* __restrict__ C, long long ldc, long long sc)
+{
+    __shared__ double As[16][65];
+    __shared__ double Bs[16][64];
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+    B += blockIdx.z * sb;
+    C += blockIdx.z * sc;
+    double acc[4][4] = {};
+    for (int k0 = 0; k0 < K; k0 += 16) {
+        for (int l = threadIdx.x; l < 1024; l += 256) {
+            const int r = l / 16, c = l % 16;
+            As[c][r] = (m0 + r < M && k0 + c < K) ? A[(long long)(m0 + r) * K + k0 + c] : 0.0;
+            const int kr = l / 64, nc = l % 64;
+            Bs[kr][nc] = (k0 + kr < K && n0 + nc < N) ? B[(long long)(k0 + kr) * ldb + n0 + nc] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+            double av[4], bv[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) av[i] = As[c][ty + 16 * i];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) bv[i] = Bs[c][tx + 16 * i];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (m0 + ty + 16 * i < M && n0 + tx + 16 * j < N) C[(long long)(m0 + ty + 16 * i) * ldc + n0 + tx + 16 * j] = acc[i][j];
+}
+
+struct EpiStore {
+    double* C;
+    long long ldc;
+    __device__ void operator()(int m, int n, double v) const { C[(long long)m * ldc + n] = v; }
+};
+
+__device__ __forceinline__ void put(double* p, double v) { *p = v; }
+__device__ __forceinline__ void put(float* p, double v) { *p = (float)v; }
+__device__ __forceinline__ void put(df32* p, double v) { *p = df_from_double(v); }
+// Columns [c0, c0 + cols) of the period-F multiplier into the plan's table (row stride ldf).
+template <class R> __global__ void k_put_columns(long long rows, int cols, const double* X, long long ldx, R* M, int c0, int ldf)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= rows * cols) return;
+    const long long r = i / cols;
+    const int c = (int)(i % cols);
+    put(M + r * ldf + c0 + c, X[r * ldx + c]);
 }
 
 inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -398,6 +493,65 @@ void sp_gs_exponents(const sp_plan p, double* a)
     for (int s = 0; s < terms; ++s) a[s] = exp(2.0 * (tau_lo + s * p->h_tau));
 }
 
+// Multiplier of the solve passes' lengths F from the 2n one (both FP64, rounded to the pass
+// type last): one contraction per axis whose length changes, 64 output columns at a time so
+// that the scratch stays at three slabs of (F0/2 + 1)(F1/2 + 1) x 64.
+static sp_status setup_period(sp_plan p, cudaStream_t st)
+{
+    const int n0p = p->n[0] + 1, n1p = p->n[1] + 1, n2p = p->n[2] + 1;
+    const int q0 = p->F[0] / 2 + 1, q1 = p->F[1] / 2 + 1, q2 = p->F[2] / 2 + 1;
+    DevBuf T0(st), T1(st), T2(st), X(st), Y(st);
+    DevBuf* T[3] = {&T0, &T1, &T2};
+    constexpr int CW = 64;
+    for (int ax = 0; ax < 3; ++ax) {
+        if (p->F[ax] == p->N[ax]) continue;
+        const long long cnt = (long long)(p->n[ax] + 1) * (p->F[ax] / 2 + 1);
+        if (T[ax]->alloc(sizeof(double) * cnt)) return sp_fail(SP_ERR_OOM, "setup: period scratch allocation failed");
+        k_period_rows<<<nblk(cnt, 256), 256, 0, st>>>(p->n[ax], p->F[ax], T[ax]->d());
+    }
+    const size_t slab = sizeof(double) * CW * (size_t)(q0 > n0p ? q0 : n0p) * (q1 > n1p ? q1 : n1p);
+    if (X.alloc(slab) || Y.alloc(slab)) return sp_fail(SP_ERR_OOM, "setup: period scratch allocation failed");
+    for (int c0 = 0; c0 < q2; c0 += CW) {
+        const int cols = q2 - c0 < CW ? q2 - c0 : CW;
+        const double* cur = p->d_M64 + c0;  // [n1p][n0p][cols], row stride ld
+        long long ld = p->ldz;
+        double* next = X.d();
+        if (T2.p) {
+            dim3 grid(1, nblk((long long)n0p * n1p, TM));
+            k_dgemm_nt<<<grid, 256, 0, st>>>(n0p * n1p, cols, n2p, p->d_M64, (long long)p->ldz,
+                                             T2.d() + (long long)c0 * n2p, (long long)n2p, EpiStore{next, CW});
+            cur = next;
+            ld = CW;
+            next = Y.d();
+        }
+        if (T0.p) {
+            dim3 grid(1, nblk(q0, 64), n1p);
+            k_dgemm_nn<<<grid, 256, 0, st>>>(q0, cols, n0p, T0.d(), cur, ld, ld * n0p, next, CW, (long long)CW * q0);
+            cur = next;
+            ld = CW;
+            next = cur == X.d() ? Y.d() : X.d();
+        }
+        if (T1.p) {  // rows (k0', column) of one k1 are contiguous, or ld apart without an earlier step
+            const long long w = (long long)q0 * ld;
+            if (ld == CW) {
+                dim3 grid(nblk(w, 64), nblk(q1, 64));
+                k_dgemm_nn<<<grid, 256, 0, st>>>(q1, (int)w, n1p, T1.d(), cur, w, 0, next, w, 0);
+            } else {
+                dim3 grid(1, nblk(q1, 64), q0);  // one k0 at a time: batch stride ld
+                k_dgemm_nn<<<grid, 256, 0, st>>>(q1, cols, n1p, T1.d(), cur, w, ld, next, (long long)CW * q0, CW);
+                ld = CW;
+            }
+            cur = next;
+        }
+        const long long rows = (long long)q0 * q1;
+        const unsigned nb = nblk(rows * cols, 256);
+        if (p->prec == SP_FP64) k_put_columns<<<nb, 256, 0, st>>>(rows, cols, cur, ld, (double*)p->d_Ms, c0, p->ldf);
+        else if (p->prec == SP_DF32) k_put_columns<<<nb, 256, 0, st>>>(rows, cols, cur, ld, (df32*)p->d_Ms, c0, p->ldf);
+        else k_put_columns<<<nb, 256, 0, st>>>(rows, cols, cur, ld, (float*)p->d_Ms, c0, p->ldf);
+    }
+    return sp_cuda_check(cudaGetLastError(), "setup: change of period");
+}
+
 sp_status sp_setup_run(sp_plan p, cudaStream_t st)
 {
     sp_status rc;
@@ -462,6 +616,19 @@ sp_status sp_setup_run(sp_plan p, cudaStream_t st)
     // K7: twiddles
     for (int ax = 0; ax < 3; ++ax) {
         k_twiddles<<<nblk(p->N[ax], 256), 256, 0, st>>>(p->N[ax], p->d_tw64[ax], p->d_tw32[ax], p->d_twdf[ax]);
+    }
+    if (p->emb) {
+        for (int ax = 0; ax < 3; ++ax) {
+            if (!p->d_twF[ax]) continue;
+            k_twiddles<<<nblk(p->F[ax], 256), 256, 0, st>>>(
+                p->F[ax], p->prec == SP_FP64 ? (cpx<double>*)p->d_twF[ax] : nullptr,
+                p->prec == SP_FP32 || p->prec == SP_MIXED ? (cpx<float>*)p->d_twF[ax] : nullptr,
+                p->prec == SP_DF32 ? (cpx<df32>*)p->d_twF[ax] : nullptr);
+        }
+        if ((rc = setup_period(p, st))) return rc;
+        rc = p->prec == SP_FP64 ? sp_embed_twiddles_f64(p, st)
+             : p->prec == SP_DF32 ? sp_embed_twiddles_df(p, st) : sp_embed_twiddles_f32(p, st);
+        if (rc) return rc;
     }
     if ((rc = sp_cuda_check(cudaGetLastError(), "twiddle kernel"))) return rc;
     if (p->prec == SP_DF32) return sp_v2_stage_twiddles_df(p, st);

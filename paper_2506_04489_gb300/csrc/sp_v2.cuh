@@ -64,7 +64,15 @@ template <class R, int N> constexpr int tw_entries() { return (tw_stage_size<R, 
 // per CTA at 512, 56 KB at 1024) limit the resident CTAs and cost a fill per CTA
 // (measured: 8 % faster at 128^3, 5 % at 256^3, 17 % at 512^3), and FP32 (its z passes
 // 20-30 % faster).  The pipelined line kernel keeps its tables in shared memory.
-template <class R, int N> constexpr bool tw_global() { return std::is_same<R, df32>::value || std::is_same<R, float>::value; }
+// The lengths of sp_embed.cuh read them from global memory in every type.
+constexpr bool len_ok(int N)
+{
+    return N == 64 || N == 128 || N == 192 || N == 256 || N == 384 || N == 512 || N == 1024;
+}
+template <class R, int N> constexpr bool tw_global()
+{
+    return std::is_same<R, df32>::value || std::is_same<R, float>::value || !len_ok(N);
+}
 template <class R, int N, class K = R> constexpr size_t pass_tw_bytes() { return tw_global<R, N>() ? 0 : sizeof(cpx<R>) * tw_entries<K, N>(); }
 
 // Offset of plan key K's staged table after an axis's N base twiddles (entries).
@@ -92,6 +100,8 @@ struct LArgs {
     int No, nh_line, ldzM;
     int reverse;                     // walk the outer index from the end: the previous pass
                                      // wrote its last outer indices last, so they are still in L2
+    int nlim;                        // grid points of the line axis (ragged passes only): rows at
+                                     // and above it are zero on input and cropped on output
 };
 
 // Largest column tile of a line pass (the launch bound of the runtime-tile kernel):
@@ -143,7 +153,9 @@ template <class R, int N, int MODE> constexpr size_t stage_m_bytes(int B) { retu
 // One tile of a line pass: B columns (c = cb B + b) of outer index o, right-hand side
 // `batch`; all threads of the block take part.  `smraw` is the pass's dynamic shared
 // memory (staged twiddles where they live in shared memory, then the exchange buffers).
-template <class R, int N, int MODE, int LGB, class K = R>
+// RAG: the axis has a.nlim <= N / 2 grid points (a transform length above twice the grid,
+// sp_embed.cuh); otherwise exactly N / 2.
+template <class R, int N, int MODE, int LGB, class K = R, bool RAG = false>
 SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smraw)
 {
     constexpr int E = PlanOf<K, N>::E, T = N / E;
@@ -178,7 +190,7 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
 #pragma unroll
         for (int j = 0; j < E; ++j) {
             const int e = first_element<K, N, false>(t, j);
-            v[j] = (cv && (j % R0) < R0 / 2) ? in[e * a.in_es] : czero<R>();
+            v[j] = (cv && (j % R0) < R0 / 2 && (!RAG || e < a.nlim)) ? in[e * a.in_es] : czero<R>();
         }
     }
     // x pass: the multiplier values of this thread's outputs are fetched before the forward
@@ -238,7 +250,8 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
     } else {  // the last inverse radix is R0: outputs q < R0/2 are the kept half
 #pragma unroll
         for (int j = 0; j < E; ++j)
-            if ((j % R0) < R0 / 2 && cv) out[last_element<K, N, true>(t, j) * a.out_es] = norm(v[j]);
+            if ((j % R0) < R0 / 2 && cv && (!RAG || last_element<K, N, true>(t, j) < a.nlim))
+                out[last_element<K, N, true>(t, j) * a.out_es] = norm(v[j]);
     }
 }
 
@@ -489,8 +502,8 @@ template <class R, int N> SP_HD bool z_two_buffers(int B)
 }
 
 // One tile of the z forward pass: a.B pairs of real lines starting at pair block `blk`,
-// right-hand side `batch`.
-template <class R, class Tio, int N>
+// right-hand side `batch`.  RAG: n2 <= N / 2 grid points a line; otherwise exactly N / 2.
+template <class R, class Tio, int N, bool RAG = false>
 SP_D void zf_tile(const ZArgs2& a, int blk, int batch, unsigned char* smraw)
 {
     constexpr int E = PlanOf<ZKey<R>, N>::E, T = N / E;
@@ -502,7 +515,7 @@ SP_D void zf_tile(const ZArgs2& a, int blk, int batch, unsigned char* smraw)
     const int tid = threadIdx.x, b = tid / T, t = tid % T;
     const cpx<R>* tws = tw_global<R, N>() ? static_cast<const cpx<R>*>(a.tw) + N : tws_s;
     if constexpr (!tw_global<R, N>()) fill_stage_twiddles<R, N, false, ZKey<R>>(tws_s, static_cast<const cpx<R>*>(a.tw), tid, blockDim.x);
-    const int n2 = a.n2;
+    const int n2 = a.n2, nh = RAG ? N / 2 : n2;
     const long long l0 = 2 * ((long long)blk * B + b), l1 = l0 + 1;
     const Tio* rho = static_cast<const Tio*>(a.rho) + batch * a.io_bs;
     cpx<R>* W = static_cast<cpx<R>*>(a.W) + batch * a.w_bs;
@@ -512,7 +525,7 @@ SP_D void zf_tile(const ZArgs2& a, int blk, int batch, unsigned char* smraw)
     for (int j = 0; j < E; ++j) {
         const int z = first_element<ZKey<R>, N, false>(t, j);
         R xr = Num<R>::c(0.0), xi = Num<R>::c(0.0);
-        if ((j % R0) < R0 / 2) {  // z < n2: the padded half is zero
+        if ((j % R0) < R0 / 2 && (!RAG || z < n2)) {  // z < n2: the padded half is zero
             if (l0 < a.lines) xr = to_r<R, Tio>(rho[l0 * n2 + z]);
             if (l1 < a.lines) xi = to_r<R, Tio>(rho[l1 * n2 + z]);
         }
@@ -524,9 +537,9 @@ SP_D void zf_tile(const ZArgs2& a, int blk, int batch, unsigned char* smraw)
     for (int j = 0; j < E; ++j) sm[lay(last_element<ZKey<R>, N, false>(t, j))] = v[j];
     __syncthreads();
     // two real lines from one complex transform: Xa = (Z_k + conj Z_{N-k}) / 2,
-    // Xb = (Z_k - conj Z_{N-k}) / (2 i), k = 0..n2
+    // Xb = (Z_k - conj Z_{N-k}) / (2 i), k = 0..N/2 = nh
     const long long r0 = w_row(a, l0), r1 = w_row(a, l1 < a.lines ? l1 : l0);
-    for (int k = t; k <= n2; k += T) {
+    for (int k = t; k <= nh; k += T) {
         const cpx<R> zk = sm[lay(k)];
         const cpx<R> zm = conjg(sm[lay(k == 0 ? 0 : N - k)]);
         const cpx<R> s = zk + zm, d = zk - zm;
@@ -544,7 +557,7 @@ __global__ void __launch_bounds__((N / PlanOf<ZKey<R>, N>::E) * pairs_max<N>(),
 }
 
 // One tile of the z inverse pass (pairs of real output lines), as zf_tile.
-template <class R, class Tio, int N>
+template <class R, class Tio, int N, bool RAG = false>
 SP_D void zi_tile(const ZArgs2& a, int blk, int batch, unsigned char* smraw)
 {
     constexpr int E = PlanOf<ZKey<R>, N>::E, T = N / E;
@@ -556,21 +569,21 @@ SP_D void zi_tile(const ZArgs2& a, int blk, int batch, unsigned char* smraw)
     const int tid = threadIdx.x, b = tid / T, t = tid % T;
     const cpx<R>* tws = tw_global<R, N>() ? static_cast<const cpx<R>*>(a.tw) + N : tws_s;
     if constexpr (!tw_global<R, N>()) fill_stage_twiddles<R, N, true, ZKey<R>>(tws_s, static_cast<const cpx<R>*>(a.tw), tid, blockDim.x);
-    const int n2 = a.n2;
+    const int n2 = a.n2, nh = RAG ? N / 2 : n2;
     const long long l0 = 2 * ((long long)blk * B + b), l1 = l0 + 1;
     Tio* u = static_cast<Tio*>(a.u) + batch * a.io_bs;
     const cpx<R>* W = static_cast<const cpx<R>*>(a.W) + batch * a.w_bs;
     const LayLine<N> lay{b * LayLine<N>::LD};
     // Z_k = Xa_k + i Xb_k from the Hermitian halves (DC and Nyquist take real parts)
     const long long r0 = w_row(a, l0), r1 = w_row(a, l1 < a.lines ? l1 : l0);
-    for (int k = t; k <= n2; k += T) {
+    for (int k = t; k <= nh; k += T) {
         const cpx<R> xa = l0 < a.lines ? W[r0 + k] : czero<R>();
         const cpx<R> xb = l1 < a.lines ? W[r1 + k] : czero<R>();
         const R ar = re_of(xa), br = re_of(xb);
-        const bool edge = k == 0 || k == n2;
+        const bool edge = k == 0 || k == nh;
         const R ai = edge ? Num<R>::c(0.0) : im_of(xa), bi = edge ? Num<R>::c(0.0) : im_of(xb);
         sm0[lay(k)] = mk(ar - bi, ai + br);
-        if (k > 0 && k < n2) sm0[lay(N - k)] = mk(ar + bi, br - ai);
+        if (k > 0 && k < nh) sm0[lay(N - k)] = mk(ar + bi, br - ai);
     }
     __syncthreads();
     cpx<R> v[E];
@@ -579,8 +592,8 @@ SP_D void zi_tile(const ZArgs2& a, int blk, int batch, unsigned char* smraw)
     run_stages<R, N, true, +1, false, ZKey<R>>(v, sm1, sm0, lay, tws, t);
 #pragma unroll
     for (int j = 0; j < E; ++j) {
-        if ((j % R0) < R0 / 2) {  // z < n2
-            const int z = last_element<ZKey<R>, N, true>(t, j);
+        const int z = last_element<ZKey<R>, N, true>(t, j);
+        if ((j % R0) < R0 / 2 && (!RAG || z < n2)) {
             if (l0 < a.lines) u[l0 * n2 + z] = from_r<R, Tio>(re_of(v[j]));
             if (l1 < a.lines) u[l1 * n2 + z] = from_r<R, Tio>(im_of(v[j]));
         }
@@ -728,11 +741,6 @@ template <class F> inline sp_status with_len(int N, F&& f)
         case 1024: return f.template run<1024>();
         default: return SP_ERR_UNSUPPORTED_SIZE;
     }
-}
-
-inline bool len_ok(int N)
-{
-    return N == 64 || N == 128 || N == 192 || N == 256 || N == 384 || N == 512 || N == 1024;
 }
 
 // variant 1: the alternative radix plan of this type and length (AltPlan), where it exists

@@ -1,9 +1,13 @@
 // v2 solve passes instantiated for double-float arithmetic (FP64 input and output,
 // passes on pairs of FP32 values, see sp_df32.cuh).
-#include "sp_v2.cuh"
+#include "sp_embed.cuh"
 
 SP_V2_LINES(extern, df32)
 SP_V2_ALT(extern, df32, 256)
+SP_F_GROUP1(SP_EMBED_DF32, extern)
+SP_F_GROUP2(SP_EMBED_DF32, extern)
+SP_F_GROUP3(SP_EMBED_DF32, extern)
+SP_F_GROUP4(SP_EMBED_DF32, extern)
 
 namespace v2 {
 template <> const void* Tabs<df32>::tw(sp_plan p, int ax) { return p->d_twdf[ax]; }
@@ -44,3 +48,11 @@ struct HasAltDF {
 }  // namespace
 
 bool sp_v2_has_alt_df(int N) { return v2::with_len(N, HasAltDF{}) == SP_OK; }
+
+sp_status sp_embed_solve_df(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st)
+{
+    return v2::solve_embed<df32, double>(p, rho, u, batch, st);
+}
+
+sp_status sp_embed_twiddles_df(sp_plan p, cudaStream_t st) { return v2::embed_twiddles<df32>(p, st); }
+sp_status sp_embed_radices_df(sp_plan p, int* out) { return v2::embed_radices<df32>(p, out); }

@@ -1,10 +1,15 @@
 // v2 solve passes instantiated for FP32 arithmetic (FP32 and mixed-precision plans).
+#include "sp_embed.cuh"
 #include "sp_plane.cuh"
 
 SP_V2_LINES(extern, float)
 SP_V2_ALT(extern, float, 256)
 SP_V2_ALT(extern, float, 512)
 SP_V2_ALT(extern, float, 1024)
+SP_F_GROUP1(SP_EMBED_FLOAT, extern)
+SP_F_GROUP2(SP_EMBED_FLOAT, extern)
+SP_F_GROUP3(SP_EMBED_FLOAT, extern)
+SP_F_GROUP4(SP_EMBED_FLOAT, extern)
 
 namespace v2 {
 template <> const void* Tabs<float>::tw(sp_plan p, int ax) { return p->d_tw32[ax]; }
@@ -90,3 +95,11 @@ struct HasAltF32 {
 }  // namespace
 
 bool sp_v2_has_alt_f32(int N) { return v2::with_len(N, HasAltF32{}) == SP_OK; }
+
+sp_status sp_embed_solve_f32(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st, bool mixed)
+{
+    return mixed ? v2::solve_embed<float, double>(p, rho, u, batch, st) : v2::solve_embed<float, float>(p, rho, u, batch, st);
+}
+
+sp_status sp_embed_twiddles_f32(sp_plan p, cudaStream_t st) { return v2::embed_twiddles<float>(p, st); }
+sp_status sp_embed_radices_f32(sp_plan p, int* out) { return v2::embed_radices<float>(p, out); }

@@ -39,15 +39,43 @@ def precision_for(accuracy: float) -> str:
     return "fp32" if accuracy >= 1e-6 else "df32"
 
 
+# Padded lengths with a tuned plan, and the transform lengths of the passes elsewhere (the
+# shortest at or above 2n): the lists of the native library.
+TUNED_LENGTHS = (64, 128, 192, 256, 384, 512, 1024)
+F_LENGTHS = (16, 32, 48, 64, 72, 80, 96, 128, 144, 160, 192, 200, 216, 256, 288, 320, 384, 400, 432, 512, 576, 640,
+             768, 864, 1024, 1280, 1536, 2048)
+
+
+def transform_length(n: int, precision: str) -> int:
+    """Transform length per axis of the solve passes of an n^3 grid (the library's rule)."""
+    N = 2 * n
+    if N in TUNED_LENGTHS:
+        return N
+    F = next(f for f in F_LENGTHS if f >= N)
+    m = N
+    for p in (2, 3, 5, 7):
+        while m % p == 0:
+            m //= p
+    limit = {"fp64": 1.8, "df32": 2.5}.get(precision, 4.0)
+    if m != 1:
+        limit *= 4.0
+    elif n <= 32:
+        limit = 4.0
+    return F if (F / N) ** 3 <= limit else N
+
+
 def entry_bytes(n: int, precision: str, max_batch: int) -> int:
     """Device bytes of one resident plan of an n^3 grid with batch buffers for max_batch
-    requests: workspace, multiplier octant and its pass-precision copy, twiddles, and the
-    input and output batch buffers (plus 1 MiB for small tables)."""
+    requests: workspace, multiplier octant and its pass-precision copy (on the octant of the
+    passes' transform length), twiddles, and the input and output batch buffers (plus 1 MiB
+    for small tables)."""
     c = 16 if precision in ("fp64", "df32") else 8
     r = 4 if precision == "fp32" else 8
     ldz = (n + 1 + 7) // 8 * 8
-    work = max_batch * c * n * 2 * n * ldz
-    tables = (n + 1) * (n + 1) * ldz * (8 + (8 if precision == "df32" else 4)) + 3 * 2 * n * 32
+    f = transform_length(n, precision)
+    ldf = (f // 2 + 1 + 7) // 8 * 8
+    work = max_batch * c * n * f * ldf
+    tables = (n + 1) * (n + 1) * ldz * 8 + (f // 2 + 1) ** 2 * ldf * (8 if precision == "df32" else 4) + 3 * 2 * n * 32
     io = 2 * max_batch * n ** 3 * r
     return work + tables + io + (1 << 20)
 
