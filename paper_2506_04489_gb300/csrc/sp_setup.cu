@@ -32,37 +32,36 @@ __global__ void k_gs_table(double tau_lo, double h, int terms, double* w, double
 }
 
 // ------------------------------------------------------------------------- K5
-// Gauss-Legendre nodes/weights on [-1, 1] by Newton's method on P_Q (one thread per
-// node).  x_i in descending order.
-__global__ void k_gauss_legendre(int Q, double* x, double* w)
+// P_Q(z) and P_{Q-1}(z) by the three-term recurrence, its rational factors as constants.
+template <int Q> __device__ __forceinline__ void legendre(double z, double& pq, double& pq1)
 {
-    int i = threadIdx.x;
+    double p0 = 1.0, p1 = z;
+#pragma unroll
+    for (int j = 1; j < Q; ++j) {
+        const double p2 = ((2.0 * j + 1.0) / (j + 1.0)) * z * p1 - (j / (j + 1.0)) * p0;
+        p0 = p1;
+        p1 = p2;
+    }
+    pq = p1;
+    pq1 = p0;
+}
+// Gauss-Legendre nodes/weights on [-1, 1] by Newton's method on P_Q (one thread per
+// node).  x_i in descending order.  The starting value is within 1e-3 and the convergence
+// quadratic: a step below 1e-9 leaves rounding alone (6 us; the 100 steps that a tolerance
+// below the rounding unit always ran took 780 us).
+template <int Q> __global__ void k_gauss_legendre(double* x, double* w)
+{
+    const int i = threadIdx.x;
     if (i >= Q) return;
-    double z = cos(kPi * (i + 0.75) / (Q + 0.5));
-    double dp = 1.0;
-    for (int it = 0; it < 100; ++it) {
-        double p0 = 1.0, p1 = z;
-        for (int j = 1; j < Q; ++j) {
-            double p2 = ((2.0 * j + 1.0) * z * p1 - j * p0) / (j + 1.0);
-            p0 = p1;
-            p1 = p2;
-        }
-        // p1 = P_Q(z), p0 = P_{Q-1}(z)
-        dp = Q * (z * p1 - p0) / (z * z - 1.0);
-        double dz = p1 / dp;
+    double z = cospi((i + 0.75) / (Q + 0.5)), p, p1;
+    for (int it = 0; it < 10; ++it) {
+        legendre<Q>(z, p, p1);
+        const double dz = p * (z * z - 1.0) / (Q * (z * p - p1));
         z -= dz;
-        if (fabs(dz) < 1e-17) break;
+        if (fabs(dz) < 1e-9) break;
     }
-    // final derivative at the converged node
-    {
-        double p0 = 1.0, p1 = z;
-        for (int j = 1; j < Q; ++j) {
-            double p2 = ((2.0 * j + 1.0) * z * p1 - j * p0) / (j + 1.0);
-            p0 = p1;
-            p1 = p2;
-        }
-        dp = Q * (z * p1 - p0) / (z * z - 1.0);
-    }
+    legendre<Q>(z, p, p1);
+    const double dp = Q * (z * p - p1) / (z * z - 1.0);
     x[i] = z;
     w[i] = 2.0 / ((1.0 - z * z) * dp * dp);
 }
@@ -133,10 +132,13 @@ __global__ void k_full_line(int s0, int terms, int nk, double L, const double* a
 }
 
 // ------------------------------------------------------------------------- GEMM
-// C[m][n] = sum_k A[m][k] B[n][k] (both operands K-contiguous), FP64, 64x64 tiles,
-// 256 threads with 4x4 outputs each, K staged through shared memory 16 at a time.
-// The epilogue functor receives (m, n, value).
-constexpr int TM = 64, TN = 64, TK = 16;
+// C[m][n] = sum_k A[m][k] B[n][k] (both operands K-contiguous), FP64, 32 x 32 tiles, 256
+// threads with 2 x 2 outputs each, K staged through shared memory 16 at a time.  Bound by the
+// FP64 pipe (two FMAs a clock an SM), so small tiles cost nothing in shared-memory reads and
+// waste less at the edges than 64 x 64 ones (129 columns: 160 instead of 192 computed; the
+// last of few waves is shorter).  The epilogue functor receives (m, n, value); skip(m0, n0)
+// names tiles that are not needed.
+constexpr int TM = 32, TN = 32, TK = 16;
 
 template <class Epi>
 __global__ void __launch_bounds__(256) k_dgemm_nt(int M, int N, int K, const double* __restrict__ A,
@@ -145,37 +147,34 @@ __global__ void __launch_bounds__(256) k_dgemm_nt(int M, int N, int K, const dou
 {
     __shared__ double As[TK][TM + 1];
     __shared__ double Bs[TK][TN + 1];
-    int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-    double acc[4][4] = {};
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+    if (epi.skip(m0, n0)) return;
+    double acc[2][2] = {};
     for (int k0 = 0; k0 < K; k0 += TK) {
+#pragma unroll
         for (int l = threadIdx.x; l < TM * TK; l += 256) {
-            int r = l / TK, c = l % TK;
-            int gm = m0 + r, gk = k0 + c;
+            const int r = l / TK, c = l % TK;
+            const int gm = m0 + r, gn = n0 + r, gk = k0 + c;
             As[c][r] = (gm < M && gk < K) ? A[(long long)gm * lda + gk] : 0.0;
-            int gn = n0 + r;
             Bs[c][r] = (gn < N && gk < K) ? B[(long long)gn * ldb + gk] : 0.0;
         }
         __syncthreads();
 #pragma unroll
         for (int c = 0; c < TK; ++c) {
-            double av[4], bv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) av[i] = As[c][ty + 16 * i];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) bv[i] = Bs[c][tx + 16 * i];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+            const double a0 = As[c][ty], a1 = As[c][ty + 16], b0 = Bs[c][tx], b1 = Bs[c][tx + 16];
+            acc[0][0] = fma(a0, b0, acc[0][0]);
+            acc[0][1] = fma(a0, b1, acc[0][1]);
+            acc[1][0] = fma(a1, b0, acc[1][0]);
+            acc[1][1] = fma(a1, b1, acc[1][1]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int gm = m0 + ty + 16 * i, gn = n0 + tx + 16 * j;
+        for (int j = 0; j < 2; ++j) {
+            const int gm = m0 + ty + 16 * i, gn = n0 + tx + 16 * j;
             if (gm < M && gn < N) epi(gm, gn, acc[i][j]);
         }
 }
@@ -188,107 +187,154 @@ __global__ void __launch_bounds__(256) k_dgemm_nt(int M, int N, int K, const dou
 // G and H have relative (not only absolute) accuracy at high wavenumber.
 __device__ __forceinline__ bool by_parts(int k, double kap, double al) { return k > 0 && kap * kap >= 4.0 * al; }
 
-struct EpiDirect {  // out[s][k] = 2 v where the direct form applies
-    double* out;
-    long long ld;
-    const double* a;
-    double L;
-    __device__ void operator()(int m, int n, double v) const
-    {
-        double kap = kPi * n / L;
-        if (!by_parts(n, kap, a[m])) out[(long long)m * ld + n] = 2.0 * v;
+// boundary terms of the by-parts form: 2 (-1)^k (P'(L)/kappa^2 - P'''(L)/kappa^4), plus 2 v / kappa^4
+// WHICH 0: P = f = exp(-a y^2); 1: P = g = y^2 exp(-a y^2)
+__device__ __forceinline__ double parts_value(int which, int k, double kap, double al, double L, double v)
+{
+    const double e = exp(-al * L * L), a2 = al * al, a3 = a2 * al, L2 = L * L;
+    double d1, d3;
+    if (which == 0) {
+        d1 = -2.0 * al * L * e;
+        d3 = (-8.0 * a3 * L2 * L + 12.0 * a2 * L) * e;
+    } else {
+        d1 = (2.0 * L - 2.0 * al * L2 * L) * e;
+        d3 = (-24.0 * al * L + 36.0 * a2 * L2 * L - 8.0 * a3 * L2 * L2 * L) * e;
     }
-};
+    const double sgn = (k & 1) ? -1.0 : 1.0, k2 = kap * kap, k4 = k2 * k2;
+    return 2.0 * (sgn * (d1 / k2 - d3 / k4) + v / k4);
+}
 
-struct EpiByParts {  // out[s][k] = 2 ((-1)^k (P'(L)/kappa^2 - P'''(L)/kappa^4) + v / kappa^4)
-    double* out;
-    long long ld;
-    const double* a;
-    double L;
-    int which;  // 0: P = f = exp(-a y^2); 1: P = g = y^2 exp(-a y^2)
-    __device__ void operator()(int m, int n, double v) const
-    {
-        double al = a[m];
-        double kap = kPi * n / L;
-        if (!by_parts(n, kap, al)) return;
-        double e = exp(-al * L * L), a2 = al * al, a3 = a2 * al, L2 = L * L;
-        double d1, d3;
-        if (which == 0) {
-            d1 = -2.0 * al * L * e;
-            d3 = (-8.0 * a3 * L2 * L + 12.0 * a2 * L) * e;
-        } else {
-            d1 = (2.0 * L - 2.0 * al * L2 * L) * e;
-            d3 = (-24.0 * al * L + 36.0 * a2 * L2 * L - 8.0 * a3 * L2 * L2 * L) * e;
+// The quadrature sums of one axis, all four (direct and by-parts integrands of G and H) in
+// one launch: 16 x 16 outputs (s, k) a block, blockIdx.z = 0 for G, 1 for H.  A block runs
+// the direct sum, the by-parts sum, or (where the border between them crosses it) both.
+// Bound by the FP64 pipe at two FMAs a clock an SM, so the tile is small: it fills the chip
+// (486 blocks at n = 128, where 64 x 64 tiles gave 21), and two shared-memory reads an FMA
+// do not show.  At n = 128 the four sums took 9.5 ms as four GEMMs.
+constexpr int kAxT = 16, kAxK = 32;
+__global__ void __launch_bounds__(kAxT * kAxT) k_axis_sums(int rows, int nk, int nq, const double* __restrict__ E,
+                                                           const double* __restrict__ C, const double* __restrict__ a, double L,
+                                                           double* __restrict__ G, double* __restrict__ H)
+{
+    __shared__ double As[kAxT][kAxK + 1], Bs[kAxT][kAxK + 1];
+    const int which = blockIdx.z, tx = threadIdx.x % kAxT, ty = threadIdx.x / kAxT;
+    const int s = blockIdx.y * kAxT + ty, k = blockIdx.x * kAxT + tx;
+    const bool in = s < rows && k < nk;
+    const double al = in ? a[s] : 1.0, kap = kPi * k / L;
+    const bool parts = in && by_parts(k, kap, al);
+    const long long rn = (long long)rows * nq;
+    for (int form = 0; form < 2; ++form) {  // 0: direct (E0, E2), 1: by parts (F0, F2)
+        if (!__syncthreads_or(in && parts == (form == 1))) continue;
+        const double* A = E + (2 * form + which) * rn;
+        double acc = 0.0;
+        for (int q0 = 0; q0 < nq; q0 += kAxK) {
+            for (int l = threadIdx.x; l < kAxT * kAxK; l += kAxT * kAxT) {
+                const int r = l / kAxK, c = l % kAxK, q = q0 + c;
+                const int gs = blockIdx.y * kAxT + r, gk = blockIdx.x * kAxT + r;
+                As[r][c] = gs < rows && q < nq ? A[(long long)gs * nq + q] : 0.0;
+                Bs[r][c] = gk < nk && q < nq ? C[(long long)gk * nq + q] : 0.0;
+            }
+            __syncthreads();
+#pragma unroll 8
+            for (int c = 0; c < kAxK; ++c) acc = fma(As[ty][c], Bs[tx][c], acc);
+            __syncthreads();
         }
-        double sgn = (n & 1) ? -1.0 : 1.0;
-        double k2 = kap * kap, k4 = k2 * k2;
-        out[(long long)m * ld + n] = 2.0 * (sgn * (d1 / k2 - d3 / k4) + v / k4);
+        if (in && parts == (form == 1)) {
+            double* out = which ? H : G;
+            out[(long long)s * nk + k] = form ? parts_value(which, k, kap, al, L, acc) : 2.0 * acc;
+        }
     }
-};
+}
 
 // ------------------------------------------------------------------------- K6
-// A'[row][c], row = k1 (n0+1) + k0 in [row0, row0 + rows):
+// Rows of the multiplier's contraction: every (k1, k0), or with SYM (axes 0 and 1 share n
+// and L, so V is symmetric in them) those with k0 <= k1, numbered k1 (k1 + 1)/2 + k0.
+__device__ __forceinline__ void mult_row(int row, int n0p, int sym, int& k0, int& k1)
+{
+    if (!sym) {
+        k1 = row / n0p;
+        k0 = row % n0p;
+        return;
+    }
+    k1 = (int)((sqrtf(8.0f * row + 1.0f) - 1.0f) * 0.5f);  // within one: corrected below
+    while (k1 * (k1 + 1) / 2 > row) --k1;
+    while ((k1 + 1) * (k1 + 2) / 2 <= row) ++k1;
+    k0 = row - k1 * (k1 + 1) / 2;
+}
+
+// Tables of one axis with the contraction index fastest: B[k][c], c < S: G[c][k], S <= c <
+// 2S: H[c - S][k].  The third axis's is the right-hand operand of the contraction, the other
+// two are read by the rows of the left-hand one.
+__global__ void k_mult_rhs(int S, int nk, const double* G, const double* H, double* B)
+{
+    const int k = blockIdx.y, c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < 2 * S) B[(long long)k * 2 * S + c] = c < S ? G[(long long)c * nk + k] : H[(long long)(c - S) * nk + k];
+}
+
+// A'[row][c], rows [row0, row0 + gridDim.y) (mult_row), from the axes' B tables:
 //   c <  S: w_c (H0[c][k0] G1[c][k1] + G0[c][k0] H1[c][k1])
 //   c >= S: w_{c-S} G0[c-S][k0] G1[c-S][k1]
-__global__ void k_mult_lhs(int row0, int rows, int S, int n0p, int n1p, const double* w,
-                           const double* G0, const double* H0, const double* G1,
-                           const double* H1, double* Ap)
+__global__ void k_mult_lhs(int row0, int S, int n0p, int sym, const double* w, const double* B0, const double* B1, double* Ap)
 {
-    long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)rows * 2 * S) return;
-    int r = (int)(idx / (2 * S)), c = (int)(idx % (2 * S));
-    int row = row0 + r;
-    int k1 = row / n0p, k0 = row % n0p;
-    int s = c < S ? c : c - S;
-    double g0 = G0[(long long)s * n0p + k0], h0 = H0[(long long)s * n0p + k0];
-    double g1 = G1[(long long)s * n1p + k1], h1 = H1[(long long)s * n1p + k1];
-    Ap[idx] = c < S ? w[s] * (h0 * g1 + g0 * h1) : w[s] * (g0 * g1);
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= 2 * S) return;
+    int k0, k1;
+    mult_row(row0 + blockIdx.y, n0p, sym, k0, k1);
+    const double *b0 = B0 + (long long)k0 * 2 * S, *b1 = B1 + (long long)k1 * 2 * S;
+    const int s = c < S ? c : c - S;
+    const double g0 = b0[s], g1 = b1[s];
+    Ap[(long long)blockIdx.y * 2 * S + c] = c < S ? w[s] * (b0[S + s] * g1 + g0 * b1[S + s]) : w[s] * (g0 * g1);
 }
 
 // Original GS method without near-field correction: A'[row][s] = 2 w_s G0 G1 (the GS of
-// 1/(4 pi r) is twice the 1/(8 pi r) table), B'[kz][s] = G2: V = sum_s 2 w_s G0 G1 G2.
-__global__ void k_plain_lhs(int row0, int rows, int S, int n0p, int n1p, const double* w,
-                            const double* G0, const double* G1, double* Ap)
+// 1/(4 pi r) is twice the 1/(8 pi r) table), contracted with the G half of the third axis's
+// table: V = sum_s 2 w_s G0 G1 G2.
+__global__ void k_plain_lhs(int row0, int S, int n0p, int sym, const double* w, const double* B0, const double* B1, double* Ap)
 {
-    long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)rows * S) return;
-    int r = (int)(idx / S), s = (int)(idx % S);
-    int row = row0 + r;
-    int k1 = row / n0p, k0 = row % n0p;
-    Ap[idx] = 2.0 * w[s] * G0[(long long)s * n0p + k0] * G1[(long long)s * n1p + k1];
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= S) return;
+    int k0, k1;
+    mult_row(row0 + blockIdx.y, n0p, sym, k0, k1);
+    Ap[(long long)blockIdx.y * S + s] = 2.0 * w[s] * B0[(long long)k0 * 2 * S + s] * B1[(long long)k1 * 2 * S + s];
 }
 
-__global__ void k_plain_rhs(int S, int n2p, const double* G2, double* Bp)
-{
-    long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)n2p * S) return;
-    int kz = (int)(idx / S), s = (int)(idx % S);
-    Bp[idx] = G2[(long long)s * n2p + kz];
-}
-
-// B'[kz][c]: c < S: G2[c][kz], c >= S: H2[c-S][kz]
-__global__ void k_mult_rhs(int S, int n2p, const double* G2, const double* H2, double* Bp)
-{
-    long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)n2p * 2 * S) return;
-    int kz = (int)(idx / (2 * S)), c = (int)(idx % (2 * S));
-    Bp[idx] = c < S ? G2[(long long)c * n2p + kz] : H2[(long long)(c - S) * n2p + kz];
-}
-
-struct EpiMultiplier {  // M[row][kz] = -(kappa0^2 + kappa1^2 + kappa2^2) V / Ntilde (or V / Ntilde)
+struct EpiMultiplier {  // M[k1][k0][kz] = -(kappa0^2 + kappa1^2 + kappa2^2) V / Ntilde (or V / Ntilde)
     double* M;
     int ldz, row0, n0p;
+    int sym, cube;      // symmetric in axes 0, 1; in all three (only kz >= k1 >= k0 is needed)
     double c0, c1, c2;  // (pi / L_p)^2
     double invN;
     int laplacian;      // 1: super-potential (spectral Laplacian applied); 0: plain GS kernel
+    // a tile is needed when its last column reaches its first row's k1 (the rows' smallest)
+    __device__ bool skip(int m0, int n0) const
+    {
+        if (!cube) return false;
+        int k0, k1;
+        mult_row(row0 + m0, n0p, sym, k0, k1);
+        return n0 + TN - 1 < k1;
+    }
     __device__ void operator()(int m, int n, double v) const
     {
-        int row = row0 + m;
-        int k1 = row / n0p, k0 = row % n0p;
-        double k2sum = c0 * (double)k0 * k0 + c1 * (double)k1 * k1 + c2 * (double)n * n;
-        M[(long long)row * ldz + n] = laplacian ? -k2sum * v * invN : v * invN;
+        int k0, k1;
+        mult_row(row0 + m, n0p, sym, k0, k1);
+        const double k2sum = c0 * (double)k0 * k0 + c1 * (double)k1 * k1 + c2 * (double)n * n;
+        const double x = laplacian ? -k2sum * v * invN : v * invN;
+        M[((long long)k1 * n0p + k0) * ldz + n] = x;
+        if (sym) M[((long long)k0 * n0p + k1) * ldz + n] = x;
     }
 };
+
+// The entries of a cube's multiplier with kz below max(k0, k1), from the sorted triple.
+__global__ void k_cube_fill(int np, int ldz, double* M)
+{
+    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (long long)np * np * np) return;
+    const int kz = (int)(idx % np), k0 = (int)(idx / np % np), k1 = (int)(idx / ((long long)np * np));
+    const int hi = k0 > k1 ? k0 : k1, lo = k0 > k1 ? k1 : k0;
+    if (kz >= hi) return;
+    // sorted: smallest and middle as (k0, k1), hi as the column
+    const int a = kz < lo ? kz : lo, b = kz < lo ? lo : kz;
+    M[((long long)k1 * np + k0) * ldz + kz] = M[((long long)b * np + a) * ldz + hi];
+}
 
 __global__ void k_to_f32(long long count, const double* in, float* out)
 {
@@ -393,6 +439,7 @@ __global__ void __launch_bounds__(256) k_dgemm_nn(int M, int N, int K, const dou
 struct EpiStore {
     double* C;
     long long ldc;
+    __device__ bool skip(int, int) const { return false; }
     __device__ void operator()(int m, int n, double v) const { C[(long long)m * ldc + n] = v; }
 };
 
@@ -439,7 +486,9 @@ static sp_status setup_axis(sp_plan p, int ax, cudaStream_t st)
             s_split, S, nk, L, p->d_gs_a, p->d_G[ax], p->d_H[ax]);
     }
     if (s_split > 0) {
-        const int P = n > 8 ? n : 8, Q = kGLQ;
+        // panels: a panel spans a phase of at most 2 pi of cos(pi k y / L), k <= n, where the
+        // 16-point rule's error is below 1e-28 of the panel's integrand
+        const int P = n > 32 ? (n + 1) / 2 : (n > 8 ? n : 8), Q = kGLQ;
         const long long nq = (long long)P * Q;
         DevBuf gl(st), nodes(st), E(st), C(st);
         const long long rn = (long long)s_split * nq;
@@ -449,19 +498,12 @@ static sp_status setup_axis(sp_plan p, int ax, cudaStream_t st)
         double *gx = gl.d(), *gw = gl.d() + Q;
         double *tpos = nodes.d(), *y = nodes.d() + nq, *wq = nodes.d() + 2 * nq;
         double *E0 = E.d(), *E2 = E0 + rn, *F0 = E2 + rn, *F2 = F0 + rn;
-        k_gauss_legendre<<<1, 32, 0, st>>>(Q, gx, gw);
+        k_gauss_legendre<kGLQ><<<1, 32, 0, st>>>(gx, gw);
         k_nodes<<<nblk(nq, 256), 256, 0, st>>>(P, Q, L, gx, gw, tpos, y, wq);
         k_gauss_rows<<<nblk(rn, 256), 256, 0, st>>>(s_split, (int)nq, p->d_gs_a, y, wq, E0, E2, F0, F2);
         k_cos_rows<<<nblk(nk * nq, 256), 256, 0, st>>>(nk, P, Q, tpos, C.d());
-        dim3 grid(nblk(nk, TN), nblk(s_split, TM));
-        k_dgemm_nt<<<grid, 256, 0, st>>>(s_split, nk, (int)nq, E0, nq, C.d(), nq,
-                                         EpiDirect{p->d_G[ax], nk, p->d_gs_a, L});
-        k_dgemm_nt<<<grid, 256, 0, st>>>(s_split, nk, (int)nq, E2, nq, C.d(), nq,
-                                         EpiDirect{p->d_H[ax], nk, p->d_gs_a, L});
-        k_dgemm_nt<<<grid, 256, 0, st>>>(s_split, nk, (int)nq, F0, nq, C.d(), nq,
-                                         EpiByParts{p->d_G[ax], nk, p->d_gs_a, L, 0});
-        k_dgemm_nt<<<grid, 256, 0, st>>>(s_split, nk, (int)nq, F2, nq, C.d(), nq,
-                                         EpiByParts{p->d_H[ax], nk, p->d_gs_a, L, 1});
+        dim3 grid(nblk(nk, kAxT), nblk(s_split, kAxT), 2);
+        k_axis_sums<<<grid, kAxT * kAxT, 0, st>>>(s_split, nk, (int)nq, E0, C.d(), p->d_gs_a, L, p->d_G[ax], p->d_H[ax]);
         rc = sp_cuda_check(cudaGetLastError(), "setup: 1D integral kernels");
         if (rc) return rc;
     }
@@ -517,7 +559,7 @@ static sp_status setup_period(sp_plan p, cudaStream_t st)
         long long ld = p->ldz;
         double* next = X.d();
         if (T2.p) {
-            dim3 grid(1, nblk((long long)n0p * n1p, TM));
+            dim3 grid(nblk(cols, TN), nblk((long long)n0p * n1p, TM));
             k_dgemm_nt<<<grid, 256, 0, st>>>(n0p * n1p, cols, n2p, p->d_M64, (long long)p->ldz,
                                              T2.d() + (long long)c0 * n2p, (long long)n2p, EpiStore{next, CW});
             cur = next;
@@ -576,17 +618,37 @@ sp_status sp_setup_run(sp_plan p, cudaStream_t st)
     // K6: multiplier, GEMM over the 2S GS columns, in row chunks
     {
         const int n0p = p->n[0] + 1, n1p = p->n[1] + 1, n2p = p->n[2] + 1;
-        const long long rows_total = (long long)n0p * n1p;
-        const int chunk = (int)(rows_total < 8192 ? rows_total : 8192);
+        // axes that share n and L make V symmetric in their wavenumbers: half of the rows where
+        // axes 0 and 1 do, and of those about a third of the columns where all three do (the
+        // rest is copied).  128^3: 2.2e6 of 16641 x 129 values are contracted three times less.
+        const bool sym = p->n[0] == p->n[1] && p->L[0] == p->L[1];
+        const bool cube = sym && p->n[1] == p->n[2] && p->L[1] == p->L[2];
+        const long long rows_total = sym ? (long long)n0p * (n0p + 1) / 2 : (long long)n0p * n1p;
+        // rows at a time: the left-hand operand of a chunk (up to 140 MB) is made just before it
+        // is read; fewer, larger chunks leave fewer partly filled last waves
         const bool plain = p->kernel == SP_KERNEL_GS_PLAIN;
         const int K = plain ? S : 2 * S;  // contraction length (GS columns)
-        DevBuf Ap(st), Bp(st);
-        if (Ap.alloc(sizeof(double) * (size_t)chunk * K) || Bp.alloc(sizeof(double) * (size_t)n2p * K))
-            return sp_fail(SP_ERR_OOM, "setup: multiplier scratch allocation failed");
-        if (plain)
-            k_plain_rhs<<<nblk((long long)n2p * S, 256), 256, 0, st>>>(S, n2p, p->d_G[2], Bp.d());
-        else
-            k_mult_rhs<<<nblk((long long)n2p * 2 * S, 256), 256, 0, st>>>(S, n2p, p->d_G[2], p->d_H[2], Bp.d());
+        long long most = (140LL << 20) / (8LL * K);
+        most = most < 256 ? 256 : (most > 16384 ? 16384 : most);
+        const int chunks = (int)((rows_total + most - 1) / most);
+        const int chunk = (int)((rows_total + chunks - 1) / chunks);
+        DevBuf Ap(st), B0(st), B1(st), B2(st);
+        DevBuf* B[3] = {&B0, &B1, &B2};
+        double* bt[3];
+        if (Ap.alloc(sizeof(double) * (size_t)chunk * K)) return sp_fail(SP_ERR_OOM, "setup: multiplier scratch allocation failed");
+        for (int ax = 0; ax < 3; ++ax) {
+            int same = ax;
+            for (int q = ax - 1; q >= 0; --q)
+                if (p->d_G[q] == p->d_G[ax]) same = q;
+            if (same < ax) {
+                bt[ax] = bt[same];
+                continue;
+            }
+            const int nk = p->n[ax] + 1;
+            if (B[ax]->alloc(sizeof(double) * (size_t)nk * 2 * S)) return sp_fail(SP_ERR_OOM, "setup: multiplier scratch allocation failed");
+            bt[ax] = B[ax]->d();
+            k_mult_rhs<<<dim3(nblk(2 * S, 256), nk), 256, 0, st>>>(S, nk, p->d_G[ax], p->d_H[ax], bt[ax]);
+        }
         EpiMultiplier epi;
         epi.M = p->d_M64;
         epi.ldz = p->ldz;
@@ -596,19 +658,20 @@ sp_status sp_setup_run(sp_plan p, cudaStream_t st)
         epi.c2 = (kPi / p->L[2]) * (kPi / p->L[2]);
         epi.invN = 1.0 / (8.0 * (double)p->n[0] * (double)p->n[1] * (double)p->n[2]);
         epi.laplacian = plain ? 0 : 1;
+        epi.sym = sym;
+        epi.cube = cube;
         for (long long r0 = 0; r0 < rows_total; r0 += chunk) {
             int rows = (int)((rows_total - r0) < chunk ? (rows_total - r0) : chunk);
             if (plain)
-                k_plain_lhs<<<nblk((long long)rows * S, 256), 256, 0, st>>>(
-                    (int)r0, rows, S, n0p, n1p, p->d_gs_w, p->d_G[0], p->d_G[1], Ap.d());
+                k_plain_lhs<<<dim3(nblk(S, 256), rows), 256, 0, st>>>((int)r0, S, n0p, sym, p->d_gs_w, bt[0], bt[1], Ap.d());
             else
-                k_mult_lhs<<<nblk((long long)rows * 2 * S, 256), 256, 0, st>>>(
-                    (int)r0, rows, S, n0p, n1p, p->d_gs_w, p->d_G[0], p->d_H[0], p->d_G[1], p->d_H[1], Ap.d());
+                k_mult_lhs<<<dim3(nblk(2 * S, 256), rows), 256, 0, st>>>((int)r0, S, n0p, sym, p->d_gs_w, bt[0], bt[1], Ap.d());
             epi.row0 = (int)r0;
             dim3 grid(nblk(n2p, TN), nblk(rows, TM));
-            k_dgemm_nt<<<grid, 256, 0, st>>>(rows, n2p, K, Ap.d(), K, Bp.d(), K, epi);
+            k_dgemm_nt<<<grid, 256, 0, st>>>(rows, n2p, K, Ap.d(), K, bt[2], 2 * S, epi);
         }
-        long long mcount = rows_total * p->ldz;
+        if (cube) k_cube_fill<<<nblk((long long)n0p * n0p * n0p, 256), 256, 0, st>>>(n0p, p->ldz, p->d_M64);
+        const long long mcount = (long long)n0p * n1p * p->ldz;
         if (p->d_M32) k_to_f32<<<nblk(mcount, 256), 256, 0, st>>>(mcount, p->d_M64, p->d_M32);
         if (p->d_Mdf) k_to_df<<<nblk(mcount, 256), 256, 0, st>>>(mcount, p->d_M64, p->d_Mdf);
         if ((rc = sp_cuda_check(cudaGetLastError(), "multiplier kernels"))) return rc;
