@@ -95,7 +95,7 @@ template <class R, int N, int MODE> sp_status rag_line(const LArgs& a, int outer
     ab.B = rag_tile<R, N>(T, rag_b_max<R, R, N>(), a.ncol, (long long)outer * batch);
     ab.lgB = 0;
     while ((1 << ab.lgB) < ab.B) ++ab.lgB;
-    const size_t buf = sizeof(cpx<R>) * LayStrided<R>::size(N, ab.B);
+    const size_t buf = sizeof(cpx<R>) * strided_size<R, R, N>(ab.B);
     const size_t twb = pass_tw_bytes<R, N, R>();
     const size_t smem = twb + (two_buffers(buf, twb) ? 2 : 1) * buf + stage_m_bytes<R, N, MODE>(ab.B);
     sp_status rc;

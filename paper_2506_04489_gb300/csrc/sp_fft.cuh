@@ -514,10 +514,11 @@ template <int RAD, int S, bool HALF, class R> SP_D void butterfly(cpx<R>* u)
 }
 
 // ------------------------------------------------------------------ stages
-// Layouts map an element index e of a line to a shared-memory slot.  They must satisfy
-// lay(e + d) = lay(e) + lay.step(d) for every d that is a multiple of 8 and every e, and
-// lay(8 j + q) = lay(8 j) + q * lay.unit for q < 8: the stage loops then compute one
-// slot per butterfly and add compile-time offsets for the others.
+// Layouts map an element index e of a line to a shared-memory slot, with padding after every
+// `per` elements (0: none): lay(e + d) = lay(e) + lay.step(d) for d a multiple of per, and
+// lay(j + q) = lay(j) + q * lay.unit where no multiple of per lies in (j, j + q].  With per
+// the transform's first radix every later stage's strides are multiples of it: the stage
+// loops compute one slot per butterfly and add compile-time offsets for the others.
 
 // Per-stage twiddle tables (in shared memory; for double-float, one copy per plan in
 // global memory): stage s (span P > 1, radix RAD) keeps w^{r k N/(P RAD)} at
@@ -567,6 +568,8 @@ template <class K, int N> constexpr bool plan_ok()
     return prod == N;
 }
 
+template <class Lay> constexpr bool steps(int d) { return Lay::per == 0 || d % (Lay::per == 0 ? 1 : Lay::per) == 0; }
+
 template <class R, int N, bool INV, int ST, class K = R> struct Stage {
     static_assert(plan_ok<K, N>(), "radix plan does not fit the stage rules");
     static constexpr int E = PlanOf<K, N>::E;
@@ -581,7 +584,7 @@ template <class R, int N, bool INV, int ST, class K = R> struct Stage {
     {
 #pragma unroll
         for (int m = 0; m < NB; ++m) {
-            if constexpr (STRIDE % 8 == 0) {
+            if constexpr (steps<Lay>(STRIDE)) {
                 const cpx<R>* p0 = sm + lay(t + T * m);
                 const int st = lay.step(STRIDE);
 #pragma unroll
@@ -633,13 +636,13 @@ template <class R, int N, bool INV, int ST, class K = R> struct Stage {
             const int i = t + T * m;
             const int k = i % P;
             const int base = (i - k) * RAD + k;
-            if constexpr (P % 8 == 0) {
+            if constexpr (P > 1 && steps<Lay>(P)) {
                 cpx<R>* p0 = sm + lay(base);
                 const int st = lay.step(P);
 #pragma unroll
                 for (int q = 0; q < RAD; ++q) p0[q * st] = v[m * RAD + q];
-            } else if constexpr (P == 1 && RAD == 8) {
-                cpx<R>* p0 = sm + lay(base);  // base = 8 i
+            } else if constexpr (P == 1 && (Lay::per == 0 || Lay::per % RAD == 0)) {
+                cpx<R>* p0 = sm + lay(base);  // base = RAD i: no padding inside the butterfly
                 const int st = lay.unit();
 #pragma unroll
                 for (int q = 0; q < RAD; ++q) p0[q * st] = v[m * RAD + q];

@@ -44,6 +44,13 @@ template <class R, int N> constexpr int plane_y_e()
     else return 1;
 }
 
+// exchange entries of the y phase
+template <class R, int N> constexpr int plane_y_size(int B)
+{
+    if constexpr (AltPlan<R, N>::exists) return strided_size<R, PlaneYKey<R, N>, N>(B);
+    else return 0;
+}
+
 template <class R, int N1, int N2> struct PlaneGeo {
     static constexpr int n1 = N1 / 2, n2 = N2 / 2;
     static constexpr int RP = n1 / kPlaneC;  // rows per CTA
@@ -56,8 +63,8 @@ template <class R, int N1, int N2> struct PlaneGeo {
     // shared memory: the stage (RP x n2 or n1 x CW complex), then one exchange buffer for
     // the z phase or the y phase, then N1 complex of scratch for the packed column
     static constexpr int STAGE = (n1 * CW > RP * n2 ? n1 * CW : RP * n2);
-    static constexpr int ZBUF = BZ * LayLine<N2>::LD;
-    static constexpr int YBUF = LayStrided<R>::size(N1, BY);
+    static constexpr int ZBUF = BZ * line_ld<ZKey<R>, N2>();
+    static constexpr int YBUF = plane_y_size<R, N1>(BY);
     static constexpr int BUF = ZBUF > YBUF ? ZBUF : YBUF;
     static constexpr size_t smem = sizeof(cpx<R>) * (size_t)(STAGE + BUF + N1);
     static constexpr bool ok = AltPlan<R, N1>::exists && tw_global<R, N1>() && tw_global<R, N2>() && n1 % (2 * kPlaneC) == 0 &&
@@ -98,7 +105,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 2) k_plane_fwd(PlaneArgs a)
     {
         const cpx<R>* tws = static_cast<const cpx<R>*>(a.twz) + N2;
         const int pb = tid / Tz, t = tid % Tz;
-        const LayLine<N2> lay{pb * LayLine<N2>::LD};
+        const LayLine<line_per<KZ, N2, false>()> lay{pb * line_ld<KZ, N2>()};
         for (int round = 0; round < RP / 2 / BZ; ++round) {
             const int y0 = r * RP + 2 * (round * BZ + pb), y1 = y0 + 1;
             cpx<R> v[EZ];
@@ -142,7 +149,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 2) k_plane_fwd(PlaneArgs a)
     {
         const cpx<R>* tws = static_cast<const cpx<R>*>(a.twy) + N1 + tw_key_offset<R, N1, KY>();
         const int b = tid & (BY - 1), t = tid >> G::LGBY;
-        const LayStrided<R> lay(G::LGBY, b);
+        const LayLines<R, KY, N1, false> lay(G::LGBY, b);
         for (int ch = 0; ch < CW / BY; ++ch) {
             const int c = ch * BY + b;
             const bool packed = r == 0 && c == 0;
@@ -200,7 +207,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 2) k_plane_inv(PlaneArgs a)
     {
         const cpx<R>* tws = static_cast<const cpx<R>*>(a.twy) + N1 + tw_key_offset<R, N1, KY>();
         const int b = tid & (BY - 1), t = tid >> G::LGBY;
-        const LayStrided<R> lay(G::LGBY, b);
+        const LayLines<R, KY, N1, true> lay(G::LGBY, b);
         for (int ch = 0; ch < CW / BY; ++ch) {
             const int c = ch * BY + b, kz = r * CW + c;
             const bool packed = r == 0 && c == 0;
@@ -233,7 +240,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 2) k_plane_inv(PlaneArgs a)
     {
         const cpx<R>* tws = static_cast<const cpx<R>*>(a.twz) + N2;
         const int pb = tid / Tz, t = tid % Tz;
-        const LayLine<N2> lay{pb * LayLine<N2>::LD};
+        const LayLine<line_per<KZ, N2, true>()> lay{pb * line_ld<KZ, N2>()};
         for (int round = 0; round < RP / 2 / BZ; ++round) {
             const int ly0 = 2 * (round * BZ + pb), ly1 = ly0 + 1;  // local rows
             __syncthreads();  // buf is free (y phase or previous round)

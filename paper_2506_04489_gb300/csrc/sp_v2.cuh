@@ -31,28 +31,58 @@ template <class R> SP_D cpx<R> half_of(cpx<R> a) { return scale(a, Num<R>::c(0.5
 
 // ------------------------------------------------------------------ layouts
 // Strided lines: lane b (column) is fastest, B = 2^lgB columns per CTA (a runtime tile,
-// handled with shifts and masks).  A padding row of B entries after every 8 rows keeps
-// the stride-8 writes of the first stage off one bank set when a row of B entries is
-// narrower than 128 bytes.
-template <class R> struct LayStrided {
+// handled with shifts and masks).  A padding row of B entries after every PER rows keeps the
+// first stage's writes, whose neighbouring threads are R0 rows apart, off one bank set when a
+// row of B entries is narrower than 128 bytes: with PER = R0 (even) the stride is R0 + 1 rows,
+// odd.  (Padding after every 8 rows, right for R0 = 8, made 16, 32 and 4 conflict two to four
+// ways: FP32 solves at 256^3 484 -> 454 us, 512^3 6.20 -> 5.99 ms, 240x180x75 203 -> 195 us,
+// double-float 64 x 128^3 13.55 -> 13.40 ms.)  An odd R0 needs no padding, and
+// the later stages' accesses run along consecutive rows.
+template <class R, int PER> struct LayStrided {
+    static constexpr int per = PER;
     int lgB, pad_mask, b;
     SP_D LayStrided(int lgB_, int b_)
         : lgB(lgB_), pad_mask(((1 << lgB_) * (int)sizeof(cpx<R>) >= 128) ? 0 : ~0), b(b_)
     {
     }
-    SP_D int operator()(int e) const { return (e << lgB) + (((e >> 3) << lgB) & pad_mask) + b; }
+    static constexpr SP_HD int pads(int e)
+    {
+        if constexpr (PER == 0) return 0;
+        else return e / PER;
+    }
+    SP_D int operator()(int e) const { return (e << lgB) + ((pads(e) << lgB) & pad_mask) + b; }
     SP_D int unit() const { return 1 << lgB; }
-    SP_D int step(int d) const { return (d << lgB) + (((d >> 3) << lgB) & pad_mask); }  // d a multiple of 8
-    static constexpr SP_HD int size(int N, int B) { return N * B + (N / 8) * (B * (int)sizeof(cpx<R>) >= 128 ? 0 : B); }
+    SP_D int step(int d) const { return (d << lgB) + ((pads(d) << lgB) & pad_mask); }  // d a multiple of PER
 };
-// Contiguous lines: lane t is fastest; one padding entry after every 8 entries.
-template <int N> struct LayLine {
-    static constexpr int LD = N + N / 8;
+// first radix of plan K's transforms (the inverse's is the forward's last)
+template <class K, int N, bool INV> constexpr int first_radix() { return radix_at<K, N, INV>(0); }
+template <class K, int N, bool INV> constexpr int strided_per()
+{
+    return first_radix<K, N, INV>() % 2 == 0 ? first_radix<K, N, INV>() : 0;
+}
+template <class R, class K, int N, bool INV> using LayLines = LayStrided<R, strided_per<K, N, INV>()>;
+// entries of an exchange buffer of B strided lines, whichever direction uses it
+template <class R, class K, int N> SP_HD constexpr int strided_size(int B)
+{
+    constexpr int f = strided_per<K, N, false>(), i = strided_per<K, N, true>();
+    constexpr int rows = (f ? N / f : 0) > (i ? N / i : 0) ? (f ? N / f : 0) : (i ? N / i : 0);
+    return N * B + (B * (int)sizeof(cpx<R>) >= 128 ? 0 : rows * B);
+}
+// Contiguous lines: lane t is fastest; one padding entry after every PER entries: 8, or the
+// first radix where it is larger (16 and 32 conflict two and four ways with 8).
+template <class K, int N, bool INV> constexpr int line_per()
+{
+    return first_radix<K, N, INV>() > 8 && first_radix<K, N, INV>() % 2 == 0 ? first_radix<K, N, INV>() : 8;
+}
+template <int PER> struct LayLine {
+    static constexpr int per = PER;
     int base;
-    SP_D int operator()(int e) const { return base + e + (e >> 3); }
+    SP_D int operator()(int e) const { return base + e + e / PER; }
     SP_D int unit() const { return 1; }
-    SP_D int step(int d) const { return d + d / 8; }
+    SP_D int step(int d) const { return d + d / PER; }  // d a multiple of PER
 };
+// entries a line takes, whichever direction uses it
+template <class K, int N> constexpr int line_ld() { return N + N / (line_per<K, N, false>() < line_per<K, N, true>() ? line_per<K, N, false>() : line_per<K, N, true>()); }
 
 // Shared memory of a pass: the staged twiddles of the directions it runs (unless they
 // are read from global memory, below), then one or two exchange buffers (two when both
@@ -160,9 +190,8 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
 {
     constexpr int E = PlanOf<K, N>::E, T = N / E;
     constexpr int R0 = PlanOf<K, N>::R[0];
-    using Lay = LayStrided<R>;
     const int lgB = LGB >= 0 ? LGB : a.lgB, B = 1 << lgB;
-    const int BUF = Lay::size(N, B);
+    const int BUF = strided_size<R, K, N>(B);
     const bool DB = two_buffers(sizeof(cpx<R>) * BUF, pass_tw_bytes<R, N, K>());
     cpx<R>* tws_s = reinterpret_cast<cpx<R>*>(smraw);
     cpx<R>* sm0 = tws_s + pass_tw_bytes<R, N, K>() / sizeof(cpx<R>);
@@ -178,7 +207,8 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
     const bool cv = c < a.ncol;
     const cpx<R>* in = static_cast<const cpx<R>*>(a.in) + batch * a.in_bs + o * a.in_os + c;
     cpx<R>* out = static_cast<cpx<R>*>(a.out) + batch * a.out_bs + o * a.out_os + c;
-    const Lay lay(lgB, b);
+    const LayLines<R, K, N, false> layf(lgB, b);
+    const LayLines<R, K, N, true> layi(lgB, b);
     cpx<R> v[E];
     if constexpr (MODE == INV) {
 #pragma unroll
@@ -224,9 +254,9 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
     __syncthreads();
     cpx<R>* fresh;
     if constexpr (MODE == INV) {
-        fresh = run_stages<R, N, true, +1, false, K>(v, sm0, sm1, lay, tws, t);
+        fresh = run_stages<R, N, true, +1, false, K>(v, sm0, sm1, layi, tws, t);
     } else {
-        fresh = run_stages<R, N, false, -1, true, K>(v, sm0, sm1, lay, tws, t);
+        fresh = run_stages<R, N, false, -1, true, K>(v, sm0, sm1, layf, tws, t);
     }
     if constexpr (MODE == XMUL) {
         if constexpr (STAGE_M) cp_async_wait_all();  // this thread's own copies: no barrier needed
@@ -241,7 +271,7 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
             }
             v[j] = scale(v[j], mv[j]);
         }
-        run_stages<R, N, true, +1, false, K>(v, fresh, fresh == sm0 ? sm1 : sm0, lay, tws, t);
+        run_stages<R, N, true, +1, false, K>(v, fresh, fresh == sm0 ? sm1 : sm0, layi, tws, t);
     }
     if constexpr (MODE == FWD) {
 #pragma unroll
@@ -303,7 +333,7 @@ template <class R, int N, int MODE, class K = R> constexpr size_t pipe_mstage_by
 template <class R, int N, int MODE, class K = R> constexpr bool pipe_two_buffers()
 {
     constexpr int B = 1 << lg_default<N>();
-    constexpr size_t buf = sizeof(cpx<R>) * (size_t)LayStrided<R>::size(N, B);
+    constexpr size_t buf = sizeof(cpx<R>) * (size_t)strided_size<R, K, N>(B);
     constexpr size_t twb = sizeof(cpx<R>) * tw_entries<K, N>();
     return !pipe_third_cta<R, N, MODE, K>() &&
            twb + 2 * buf + sizeof(cpx<R>) * (size_t)stage_rows<R, N, MODE>() * B <= 110 * 1024;
@@ -311,7 +341,7 @@ template <class R, int N, int MODE, class K = R> constexpr bool pipe_two_buffers
 template <class R, int N, int MODE, class K = R> constexpr size_t pipe_smem()
 {
     constexpr int B = 1 << lg_default<N>();
-    constexpr size_t buf = sizeof(cpx<R>) * (size_t)LayStrided<R>::size(N, B);
+    constexpr size_t buf = sizeof(cpx<R>) * (size_t)strided_size<R, K, N>(B);
     constexpr size_t twb = sizeof(cpx<R>) * tw_entries<K, N>();
     return twb + (pipe_two_buffers<R, N, MODE, K>() ? 2 : 1) * buf + sizeof(cpx<R>) * (size_t)stage_rows<R, N, MODE>() * B +
            pipe_mstage_bytes<R, N, MODE, K>();
@@ -327,17 +357,16 @@ __global__ void __launch_bounds__(line_threads<R, N, lg_default<N>(), K>(),
     constexpr int LGB = lg_default<N>(), B = 1 << LGB;
     constexpr int NIN = stage_rows<R, N, MODE>();
     constexpr int CH = B * (int)sizeof(cpx<R>) / 16;  // 16-byte chunks per row
-    using Lay = LayStrided<R>;
     constexpr bool MST = pipe_mstage<R, N, MODE, K>();
     constexpr int MROWS = N / 2 + 1;              // MST: multiplier rows |kx| = 0 .. N/2
     constexpr int MCH = B * (int)sizeof(R) / 16;  // MST: 16-byte chunks per multiplier row
     // cp.async writes 16-byte chunks: the stage must start on a 16-byte boundary
     static_assert((sizeof(cpx<R>) * tw_entries<K, N>()) % 16 == 0, "twiddle area alignment");
-    static_assert((sizeof(cpx<R>) * Lay::size(N, B)) % 16 == 0, "exchange buffer alignment");
+    static_assert((sizeof(cpx<R>) * strided_size<R, K, N>(B)) % 16 == 0, "exchange buffer alignment");
     static_assert((B * sizeof(cpx<R>)) % 16 == 0, "stage row alignment");
     static_assert(!MST || (B * sizeof(R)) % 16 == 0, "multiplier stage alignment");
     const LArgs& a = pa.a;
-    const int BUF = Lay::size(N, B);
+    const int BUF = strided_size<R, K, N>(B);
     constexpr bool DB = pipe_two_buffers<R, N, MODE, K>();
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<R>* tws = reinterpret_cast<cpx<R>*>(smraw);
@@ -349,7 +378,8 @@ __global__ void __launch_bounds__(line_threads<R, N, lg_default<N>(), K>(),
     const cpx<R>* twg = static_cast<const cpx<R>*>(a.tw);
     if constexpr (MODE != INV) fill_stage_twiddles<R, N, false, K>(tws, twg, tid, blockDim.x);
     if constexpr (MODE != FWD) fill_stage_twiddles<R, N, true, K>(tws, twg, tid, blockDim.x);
-    const Lay lay(LGB, b);
+    const LayLines<R, K, N, false> layf(LGB, b);
+    const LayLines<R, K, N, true> layi(LGB, b);
     // tile index = (batch * outer + o) * ncb + cb.  The first tile is decoded by division;
     // each later one adds gridDim.x in that mixed radix (two compares, no division).
     struct TileIdx {
@@ -431,9 +461,9 @@ __global__ void __launch_bounds__(line_threads<R, N, lg_default<N>(), K>(),
         if (tile + (int)gridDim.x < pa.ntiles) issue(nxt);
         cpx<R>* fresh;
         if constexpr (MODE == INV) {
-            fresh = run_stages<R, N, true, +1, false, K>(v, sm0, sm1, lay, tws, t);
+            fresh = run_stages<R, N, true, +1, false, K>(v, sm0, sm1, layi, tws, t);
         } else {
-            fresh = run_stages<R, N, false, -1, true, K>(v, sm0, sm1, lay, tws, t);
+            fresh = run_stages<R, N, false, -1, true, K>(v, sm0, sm1, layf, tws, t);
         }
         if constexpr (MODE == XMUL) {
 #pragma unroll
@@ -456,7 +486,7 @@ __global__ void __launch_bounds__(line_threads<R, N, lg_default<N>(), K>(),
                     cp_async_commit();
                 }
             }
-            run_stages<R, N, true, +1, false, K>(v, fresh, fresh == sm0 ? sm1 : sm0, lay, tws, t);
+            run_stages<R, N, true, +1, false, K>(v, fresh, fresh == sm0 ? sm1 : sm0, layi, tws, t);
         }
         cpx<R>* out = static_cast<cpx<R>*>(a.out) + batch * a.out_bs + o * a.out_os + c;
         if constexpr (MODE == FWD) {
@@ -495,7 +525,7 @@ template <int N> constexpr int pairs_default() { return N >= 512 ? 4 : (N >= 256
 
 SP_D long long w_row(const ZArgs2& a, long long l) { return (l / a.n1) * a.plane + (l % a.n1) * a.ldz; }
 
-template <class R, int N> SP_HD int z_buf(int B) { return B * LayLine<N>::LD; }
+template <class R, int N> SP_HD int z_buf(int B) { return B * line_ld<ZKey<R>, N>(); }
 template <class R, int N> SP_HD bool z_two_buffers(int B)
 {
     return two_buffers(sizeof(cpx<R>) * z_buf<R, N>(B), pass_tw_bytes<R, N, ZKey<R>>());
@@ -519,7 +549,7 @@ SP_D void zf_tile(const ZArgs2& a, int blk, int batch, unsigned char* smraw)
     const long long l0 = 2 * ((long long)blk * B + b), l1 = l0 + 1;
     const Tio* rho = static_cast<const Tio*>(a.rho) + batch * a.io_bs;
     cpx<R>* W = static_cast<cpx<R>*>(a.W) + batch * a.w_bs;
-    const LayLine<N> lay{b * LayLine<N>::LD};
+    const LayLine<line_per<ZKey<R>, N, false>()> lay{b * line_ld<ZKey<R>, N>()};
     cpx<R> v[E];
 #pragma unroll
     for (int j = 0; j < E; ++j) {
@@ -573,7 +603,7 @@ SP_D void zi_tile(const ZArgs2& a, int blk, int batch, unsigned char* smraw)
     const long long l0 = 2 * ((long long)blk * B + b), l1 = l0 + 1;
     Tio* u = static_cast<Tio*>(a.u) + batch * a.io_bs;
     const cpx<R>* W = static_cast<const cpx<R>*>(a.W) + batch * a.w_bs;
-    const LayLine<N> lay{b * LayLine<N>::LD};
+    const LayLine<line_per<ZKey<R>, N, true>()> lay{b * line_ld<ZKey<R>, N>()};
     // Z_k = Xa_k + i Xb_k from the Hermitian halves (DC and Nyquist take real parts)
     const long long r0 = w_row(a, l0), r1 = w_row(a, l1 < a.lines ? l1 : l0);
     for (int k = t; k <= nh; k += T) {
@@ -637,7 +667,7 @@ sp_status launch_line(const LArgs& a, int outer, int batch, cudaStream_t st)
     if (B < 1 || B > lanes_b_max<R, N>() || (B & (B - 1))) return sp_fail(SP_ERR_INVALID, "bad line tile %d", B);
     ab.lgB = 0;
     while ((1 << ab.lgB) < B) ++ab.lgB;
-    const size_t buf = sizeof(cpx<R>) * LayStrided<R>::size(N, B);
+    const size_t buf = sizeof(cpx<R>) * strided_size<R, K, N>(B);
     const size_t twb = pass_tw_bytes<R, N, K>();
     const size_t smem = twb + (two_buffers(buf, twb) ? 2 : 1) * buf + stage_m_bytes<R, N, MODE>(B);
     dim3 grid((unsigned)((a.ncol + B - 1) / B), (unsigned)outer, (unsigned)batch);
@@ -1028,10 +1058,10 @@ template <class R, int N> constexpr bool persist_ok()
 template <class R, int N> constexpr size_t persist_smem()
 {
     constexpr int B = 1 << persist_lgb<R, N>();
-    constexpr size_t lbuf = sizeof(cpx<R>) * (size_t)LayStrided<R>::size(N, B);
+    constexpr size_t lbuf = sizeof(cpx<R>) * (size_t)strided_size<R, R, N>(B);
     constexpr size_t ltw = pass_tw_bytes<R, N>();
     constexpr size_t line = ltw + (two_buffers(lbuf, ltw) ? 2 : 1) * lbuf + stage_m_bytes<R, N, XMUL>(B);
-    constexpr size_t zbuf = sizeof(cpx<R>) * (size_t)persist_bz<R, N>() * LayLine<N>::LD;
+    constexpr size_t zbuf = sizeof(cpx<R>) * (size_t)persist_bz<R, N>() * line_ld<ZKey<R>, N>();
     constexpr size_t ztw = pass_tw_bytes<R, N, ZKey<R>>();
     constexpr size_t zs = ztw + (two_buffers(zbuf, ztw) ? 2 : 1) * zbuf;
     return line > zs ? line : zs;
