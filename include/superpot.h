@@ -147,7 +147,7 @@ sp_status sp_plan_set_kernel(sp_plan plan, sp_kernel kind);
 /*
  * sp_kernel_precompute -- Alg. 1 on the GPU, all in FP64: GS table (if not given),
  * the 1D integral tables G, H of eq. (Gten_sep) (closed full-line forms where
- * a_s L^2 >= 40; else composite 16-point Gauss-Legendre with nodes computed on the
+ * a_s L^2 >= 40; else composite 16-point Gauss-Legendre with tabulated nodes on the
  * device, applied directly for kappa^2 < 4 a_s and, above, to the fourth-derivative
  * remainder after two exact integrations by parts), the multiplier M_k of
  * eq. (convtheorem), and the FFT twiddles.

@@ -32,52 +32,26 @@ __global__ void k_gs_table(double tau_lo, double h, int terms, double* w, double
 }
 
 // ------------------------------------------------------------------------- K5
-// P_Q(z) and P_{Q-1}(z) by the three-term recurrence, its rational factors as constants.
-template <int Q> __device__ __forceinline__ void legendre(double z, double& pq, double& pq1)
-{
-    double p0 = 1.0, p1 = z;
-#pragma unroll
-    for (int j = 1; j < Q; ++j) {
-        const double p2 = ((2.0 * j + 1.0) / (j + 1.0)) * z * p1 - (j / (j + 1.0)) * p0;
-        p0 = p1;
-        p1 = p2;
-    }
-    pq = p1;
-    pq1 = p0;
-}
-// Gauss-Legendre nodes/weights on [-1, 1] by Newton's method on P_Q (one thread per
-// node).  x_i in descending order.  The starting value is within 1e-3 and the convergence
-// quadratic: a step below 1e-9 leaves rounding alone (6 us; the 100 steps that a tolerance
-// below the rounding unit always ran took 780 us).
-template <int Q> __global__ void k_gauss_legendre(double* x, double* w)
-{
-    const int i = threadIdx.x;
-    if (i >= Q) return;
-    double z = cospi((i + 0.75) / (Q + 0.5)), p, p1;
-    for (int it = 0; it < 10; ++it) {
-        legendre<Q>(z, p, p1);
-        const double dz = p * (z * z - 1.0) / (Q * (z * p - p1));
-        z -= dz;
-        if (fabs(dz) < 1e-9) break;
-    }
-    legendre<Q>(z, p, p1);
-    const double dp = Q * (z * p - p1) / (z * z - 1.0);
-    x[i] = z;
-    w[i] = 2.0 / ((1.0 - z * z) * dp * dp);
-}
+// Gauss-Legendre nodes and weights of 16 points on [-1, 1], the positive half in descending
+// order: the roots of P_16 and 2 (1 - x^2)/(16 P_15(x))^2, evaluated to 50 digits and rounded
+// (Newton's method in FP64 left 3e-16 on the weights' sum, a common factor of G and H).
+__constant__ double kGlX[kGLQ / 2] = {0.9894009349916499326, 0.94457502307323257608, 0.86563120238783174388, 0.7554044083550030339,
+                                      0.61787624440264374845, 0.45801677765722738634, 0.28160355077925891323, 0.095012509837637440185};
+__constant__ double kGlW[kGLQ / 2] = {0.027152459411754094852, 0.062253523938647892863, 0.09515851168249278481, 0.12462897125553387205,
+                                      0.14959598881657673208, 0.16915651939500253819, 0.18260341504492358887, 0.18945061045506849629};
 
 // Quadrature nodes of the composite rule: P panels of Q points on [0, L].
 // t[j] = (panel + (1 + x_i)/2) position in units of the panel width, wq[j] = weight.
-__global__ void k_nodes(int P, int Q, double L, const double* gx, const double* gw,
-                        double* tpos, double* y, double* wq)
+__global__ void k_nodes(int P, double L, double* tpos, double* y, double* wq)
 {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= P * Q) return;
-    int panel = j / Q, i = j % Q;
-    double t = 0.5 * (1.0 + gx[i]);
+    if (j >= P * kGLQ) return;
+    int panel = j / kGLQ, i = j % kGLQ;
+    const int h = i < kGLQ / 2 ? i : kGLQ - 1 - i;
+    double t = 0.5 * (1.0 + (i < kGLQ / 2 ? kGlX[h] : -kGlX[h]));
     tpos[j] = t;
     y[j] = L * (panel + t) / P;
-    wq[j] = 0.5 * (L / P) * gw[i];
+    wq[j] = 0.5 * (L / P) * kGlW[h];
 }
 
 // Quadrature weights times the integrands, per GS row s and node j:
@@ -234,8 +208,10 @@ __global__ void __launch_bounds__(kAxT * kAxT) k_axis_sums(int rows, int nk, int
                 Bs[r][c] = gk < nk && q < nq ? C[(long long)gk * nq + q] : 0.0;
             }
             __syncthreads();
+            double part = 0.0;  // summed by steps: the rounding of nq terms in a row stays below the rule's
 #pragma unroll 8
-            for (int c = 0; c < kAxK; ++c) acc = fma(As[ty][c], Bs[tx][c], acc);
+            for (int c = 0; c < kAxK; ++c) part = fma(As[ty][c], Bs[tx][c], part);
+            acc += part;
             __syncthreads();
         }
         if (in && parts == (form == 1)) {
@@ -490,16 +466,14 @@ static sp_status setup_axis(sp_plan p, int ax, cudaStream_t st)
         // 16-point rule's error is below 1e-28 of the panel's integrand
         const int P = n > 32 ? (n + 1) / 2 : (n > 8 ? n : 8), Q = kGLQ;
         const long long nq = (long long)P * Q;
-        DevBuf gl(st), nodes(st), E(st), C(st);
+        DevBuf nodes(st), E(st), C(st);
         const long long rn = (long long)s_split * nq;
-        if (gl.alloc(sizeof(double) * 2 * Q) || nodes.alloc(sizeof(double) * 3 * nq) ||
+        if (nodes.alloc(sizeof(double) * 3 * nq) ||
             E.alloc(sizeof(double) * 4 * rn) || C.alloc(sizeof(double) * nk * nq))
             return sp_fail(SP_ERR_OOM, "setup: quadrature scratch allocation failed");
-        double *gx = gl.d(), *gw = gl.d() + Q;
         double *tpos = nodes.d(), *y = nodes.d() + nq, *wq = nodes.d() + 2 * nq;
         double *E0 = E.d(), *E2 = E0 + rn, *F0 = E2 + rn, *F2 = F0 + rn;
-        k_gauss_legendre<kGLQ><<<1, 32, 0, st>>>(gx, gw);
-        k_nodes<<<nblk(nq, 256), 256, 0, st>>>(P, Q, L, gx, gw, tpos, y, wq);
+        k_nodes<<<nblk(nq, 256), 256, 0, st>>>(P, L, tpos, y, wq);
         k_gauss_rows<<<nblk(rn, 256), 256, 0, st>>>(s_split, (int)nq, p->d_gs_a, y, wq, E0, E2, F0, F2);
         k_cos_rows<<<nblk(nk * nq, 256), 256, 0, st>>>(nk, P, Q, tpos, C.d());
         dim3 grid(nblk(nk, kAxT), nblk(s_split, kAxT), 2);
