@@ -80,10 +80,10 @@ template <int E_, int... Rs> struct PlanE : Radices<Rs...> {
 // prunes it uniformly), then 3s.  E is a multiple of every radix.
 template <int N> struct FFTPlan;
 template <> struct FFTPlan<64> { static constexpr int NS = 2, E = 8; static constexpr int R[2] = {8, 8}; };
-template <> struct FFTPlan<128> { static constexpr int NS = 3, E = 8; static constexpr int R[3] = {8, 8, 2}; };
-template <> struct FFTPlan<192> { static constexpr int NS = 3, E = 24; static constexpr int R[3] = {8, 8, 3}; };
+template <> struct FFTPlan<128> : PlanE<8, 8, 4, 4> {};
+template <> struct FFTPlan<192> : PlanE<12, 12, 4, 4> {};
 template <> struct FFTPlan<256> { static constexpr int NS = 3, E = 8; static constexpr int R[3] = {8, 8, 4}; };
-template <> struct FFTPlan<384> { static constexpr int NS = 4, E = 24; static constexpr int R[4] = {8, 8, 2, 3}; };
+template <> struct FFTPlan<384> : PlanE<12, 12, 4, 4, 2> {};
 template <> struct FFTPlan<512> { static constexpr int NS = 3, E = 8; static constexpr int R[3] = {8, 8, 8}; };
 template <> struct FFTPlan<1024> { static constexpr int NS = 4, E = 8; static constexpr int R[4] = {8, 8, 8, 2}; };
 
@@ -95,13 +95,13 @@ struct Plan1024Radix16 {
     static constexpr int NS = 3, E = 16;
     static constexpr int R[3] = {16, 8, 8};
 };
-// At 384, 24 double-float values a thread hold too many registers: double-float takes
-// radices 4-4-4-2-3 with 12 values a thread (7 % faster at 192^3); FP32 and FP64 keep
-// 8-8-2-3 (measured faster for them).
-struct Plan384Radix4 {
-    static constexpr int NS = 5, E = 12;
-    static constexpr int R[5] = {4, 4, 4, 2, 3};
-};
+// Lengths with a factor 3 run 12-point first stages on 12 values a thread (x passes, ps a
+// point: at 192 12-4-4 against 8-8-3 on 24 values, double-float 15.4 against 21.2, FP64 77
+// against 87, FP32 4.7 against 5.1; at 384 12-4-4-2 against 4-4-4-2-3, double-float 19.9
+// against 23.8); FP32 takes 8-8-6 on 24 values at 384.  At 128 8-4-4 (11.4 against 11.9 for
+// 8-8-2); FP32 16-8.
+struct Plan384Radix6 : PlanE<24, 8, 8, 6> {};
+struct Plan128Radix16 : PlanE<16, 16, 8> {};
 // At 256, FP32 takes two radix-16 stages (16 values a thread, one exchange instead of
 // two: 128^3 FP32 solve 12 % faster); the 16-byte types keep 8-8-4.
 struct Plan256Radix16 {
@@ -125,7 +125,8 @@ struct Plan1024Radix32 {
 };
 template <> struct PlanOf<float, 1024> : Plan1024Radix32 {};
 template <> struct PlanOf<double, 1024> : Plan1024Radix16 {};
-template <> struct PlanOf<df32, 384> : Plan384Radix4 {};
+template <> struct PlanOf<float, 384> : Plan384Radix6 {};
+template <> struct PlanOf<float, 128> : Plan128Radix16 {};
 // Lengths of the passes on grids whose own padded length has no plan above (sp_embed.cuh).
 // First radices of 4, 6, 8, 10, 12, 16 or 20 points, so that the zero half is pruned; the
 // radices 6 to 20 are prime-factor products without inner twiddles.  Plans were chosen by
