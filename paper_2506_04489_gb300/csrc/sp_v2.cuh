@@ -141,7 +141,21 @@ template <class R, int N> constexpr int lanes_b_max()
 {
     return sizeof(cpx<R>) >= 16 ? (N >= 1024 ? 4 : 8) : (N >= 1024 ? 8 : 16);
 }
-template <int N> constexpr int lanes_b_default() { return N >= 1024 ? 4 : 8; }
+// Column tile of a plan that was not tuned.  16-byte values: smaller CTAs wait less at their
+// barriers and balance better, down to where half-used sectors and idle lanes cost more.
+// Double-float 4 columns, FP64 2 from 128 up (x passes, us, 8 columns against this: double-
+// float 128^3 129 / 117, 256^3 1065 / 1003, FP64 32^3 20.8 / 16.5, 128^3 788 / 745, 256^3
+// 7034 / 6536); at 1024 (4 at most) the x pass takes 2 (512^3 14.2 / 12.8 ms) and the
+// double-float y passes at 512 stay at 8 (293/282 against 306/299).  FP32: 8 columns, the
+// pipelined kernel's tile; at 1024 its x pass is faster without the pipeline on 8 (16 warps
+// an SM and whole sectors) than with it on 4 (8 warps): 512^3 3.65 / 2.89 ms.
+template <class R, int N, int MODE> constexpr int lanes_b_default()
+{
+    if (std::is_same<R, float>::value) return N >= 1024 && MODE != XMUL ? 4 : 8;
+    if (N >= 1024) return MODE == XMUL ? 2 : 4;
+    if (std::is_same<R, double>::value) return N >= 128 ? 2 : 4;
+    return N >= 512 && MODE != XMUL ? 8 : 4;
+}
 
 // Resident CTAs per SM requested from the compiler: 1024 threads per SM (at most 64
 // registers per thread) for the 8-value plans, to hide global-memory latency; the
@@ -521,7 +535,15 @@ struct ZArgs2 {
 };
 
 template <int N> constexpr int pairs_max() { return N >= 512 ? 8 : (N >= 256 ? 16 : 32); }
-template <int N> constexpr int pairs_default() { return N >= 512 ? 4 : (N >= 256 ? 8 : 16); }
+// Pairs of a z-pass CTA of a plan that was not tuned: 64 threads (128 for FP32 at eight
+// values a thread), so that few lines share a barrier (z forward/inverse, us, 4 to 16 pairs
+// against this: double-float 128^3 34/31 / 31/28, 256^3 184/184 / 167/161, 192^3 99/103 /
+// 82/84; FP32 256^3 58/60 / 53/56, 512^3 386/575 / 335/518).
+template <class R, int N> constexpr int pairs_default()
+{
+    constexpr int E = PlanOf<ZKey<R>, N>::E, T = N / E, threads = std::is_same<R, float>::value && E <= 8 ? 128 : 64;
+    return T >= threads ? 1 : threads / T;
+}
 
 SP_D long long w_row(const ZArgs2& a, long long l) { return (l / a.n1) * a.plane + (l % a.n1) * a.ldz; }
 
@@ -662,7 +684,7 @@ sp_status launch_line(const LArgs& a, int outer, int batch, cudaStream_t st)
 {
     constexpr int E = PlanOf<K, N>::E;
     LArgs ab = a;
-    ab.B = a.B ? a.B : lanes_b_default<N>();
+    ab.B = a.B ? a.B : lanes_b_default<R, N, MODE>();
     const int B = ab.B;
     if (B < 1 || B > lanes_b_max<R, N>() || (B & (B - 1))) return sp_fail(SP_ERR_INVALID, "bad line tile %d", B);
     ab.lgB = 0;
@@ -715,7 +737,7 @@ sp_status launch_z(const ZArgs2& a, bool forward, int batch, cudaStream_t st)
 {
     constexpr int E = PlanOf<ZKey<R>, N>::E;
     ZArgs2 ab = a;
-    ab.B = a.B ? a.B : pairs_default<N>();
+    ab.B = a.B ? a.B : pairs_default<R, N>();
     const int B = ab.B;
     if (B < 1 || B > pairs_max<N>() || (pairs_max<N>() % B)) return sp_fail(SP_ERR_INVALID, "bad z tile %d", B);
     const size_t smem = pass_tw_bytes<R, N, ZKey<R>>() + sizeof(cpx<R>) * (z_two_buffers<R, N>(B) ? 2 : 1) * z_buf<R, N>(B);
