@@ -41,6 +41,7 @@ __global__ void __launch_bounds__((N / PlanOf<R, N>::E) * rag_b_max<R, R, N>(),
                                   rag_min_blocks<R, R, N>((N / PlanOf<R, N>::E) * rag_b_max<R, R, N>())) k_rag_line(LArgs a)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
+    grid_dependency();
     line_tile<R, N, MODE, -1, R, true>(a, blockIdx.x, a.reverse ? gridDim.y - 1 - blockIdx.y : blockIdx.y, blockIdx.z, smraw);
 }
 
@@ -55,6 +56,7 @@ __global__ void __launch_bounds__((N / PlanOf<ZKey<R>, N>::E) * rag_pairs_max<R,
     k_rag_z(ZArgs2 a)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
+    grid_dependency();
     const int blk = a.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
     if constexpr (FORWARD) zf_tile<R, Tio, N, true>(a, blk, blockIdx.y, smraw);
     else zi_tile<R, Tio, N, true>(a, blk, blockIdx.y, smraw);
@@ -101,8 +103,7 @@ template <class R, int N, int MODE> sp_status rag_line(const LArgs& a, int outer
     sp_status rc;
     if ((rc = smem_attr<k_rag_line<R, N, MODE>>(smem))) return rc;
     dim3 grid((unsigned)((a.ncol + ab.B - 1) / ab.B), (unsigned)outer, (unsigned)batch);
-    k_rag_line<R, N, MODE><<<grid, T * ab.B, smem, st>>>(ab);
-    return sp_cuda_check(cudaGetLastError(), "ragged line pass");
+    return launch_pass(k_rag_line<R, N, MODE>, grid, T * ab.B, smem, st, ab, a.dependent != 0, "ragged line pass");
 }
 
 template <class R, class Tio, int N> sp_status rag_z(const ZArgs2& a, bool forward, int batch, cudaStream_t st)
@@ -116,12 +117,11 @@ template <class R, class Tio, int N> sp_status rag_z(const ZArgs2& a, bool forwa
     sp_status rc;
     if (forward) {
         if ((rc = smem_attr<k_rag_z<R, Tio, N, true>>(smem))) return rc;
-        k_rag_z<R, Tio, N, true><<<grid, T * ab.B, smem, st>>>(ab);
+        return launch_pass(k_rag_z<R, Tio, N, true>, grid, T * ab.B, smem, st, ab, a.dependent != 0, "ragged z forward pass");
     } else {
         if ((rc = smem_attr<k_rag_z<R, Tio, N, false>>(smem))) return rc;
-        k_rag_z<R, Tio, N, false><<<grid, T * ab.B, smem, st>>>(ab);
+        return launch_pass(k_rag_z<R, Tio, N, false>, grid, T * ab.B, smem, st, ab, a.dependent != 0, "ragged z inverse pass");
     }
-    return sp_cuda_check(cudaGetLastError(), forward ? "ragged z forward pass" : "ragged z inverse pass");
 }
 
 // Calls f.template run<F>() for a listed length F.
@@ -195,6 +195,7 @@ template <class R, class Tio> sp_status solve_embed(sp_plan p, const void* rho, 
     z.io_bs = (long long)p->n[0] * p->n[1] * p->n[2];
     z.w_bs = (long long)p->n[0] * p->planef;
     z.tw = embed_tw<R>(p, 2);
+    z.dependent = (size_t)batch * z.w_bs * sizeof(cpx<R>) <= kDependentBytes;
     LArgs y = {};
     y.in = y.out = p->d_work;
     y.in_os = y.out_os = p->planef;
@@ -204,6 +205,7 @@ template <class R, class Tio> sp_status solve_embed(sp_plan p, const void* rho, 
     y.in_ld = p->ldf;
     y.tw = embed_tw<R>(p, 1);
     y.nlim = p->n[1];
+    y.dependent = z.dependent;
     LArgs x = y;
     x.in_os = x.out_os = p->ldf;
     x.in_es = x.out_es = p->planef;
