@@ -31,7 +31,7 @@ template <class R, class K, int N> constexpr int rag_b_max()
 template <class R, class K, int N> constexpr int rag_min_blocks(int threads)
 {
     constexpr int E = PlanOf<K, N>::E, T = N / E;
-    constexpr int cap = sizeof(cpx<R>) >= 16 ? (E <= 6 ? 96 : (E >= 12 && T < 64 ? 168 : 128)) : (E <= 8 ? 64 : (E <= 16 ? 96 : (E <= 24 ? 128 : 168)));
+    constexpr int cap = sizeof(cpx<R>) >= 16 ? (E <= 6 ? 96 : (E >= 12 && T < 64 ? 168 : 128)) : (E <= 8 ? 64 : (E <= 16 ? 96 : 128));
     const int b = 65536 / (cap * threads);
     return b < 1 ? 1 : b;
 }
@@ -97,9 +97,7 @@ template <class R, int N, int MODE> sp_status rag_line(const LArgs& a, int outer
     ab.B = rag_tile<R, N>(T, rag_b_max<R, R, N>(), a.ncol, (long long)outer * batch);
     ab.lgB = 0;
     while ((1 << ab.lgB) < ab.B) ++ab.lgB;
-    const size_t buf = sizeof(cpx<R>) * strided_size<R, R, N>(ab.B);
-    const size_t twb = pass_tw_bytes<R, N, R>();
-    const size_t smem = twb + (two_buffers(buf, twb) ? 2 : 1) * buf + stage_m_bytes<R, N, MODE>(ab.B);
+    const size_t smem = line_smem<R, N, MODE>(ab.B);
     sp_status rc;
     if ((rc = smem_attr<k_rag_line<R, N, MODE>>(smem))) return rc;
     dim3 grid((unsigned)((a.ncol + ab.B - 1) / ab.B), (unsigned)outer, (unsigned)batch);

@@ -187,11 +187,12 @@ template <class R, int N> constexpr int lanes_b_max()
 // float 128^3 129 / 117, 256^3 1065 / 1003, FP64 32^3 20.8 / 16.5, 128^3 788 / 745, 256^3
 // 7034 / 6536); at 1024 (4 at most) the x pass takes 2 (512^3 14.2 / 12.8 ms) and the
 // double-float y passes at 512 stay at 8 (293/282 against 306/299).  FP32: 8 columns, the
-// pipelined kernel's tile; at 1024 its x pass is faster without the pipeline on 8 (16 warps
-// an SM and whole sectors) than with it on 4 (8 warps): 512^3 3.65 / 2.89 ms.
+// pipelined kernel's tile; at 1024 the x and y forward passes are faster without the pipeline
+// on 8 (16 warps an SM, 64-byte rows) than with it on 4 (8 warps): 512^3 x 3.66 / 1.96 ms, y
+// forward 0.69 / 0.64, y inverse 0.70 / 0.71.
 template <class R, int N, int MODE> constexpr int lanes_b_default()
 {
-    if (std::is_same<R, float>::value) return N >= 1024 && MODE != XMUL ? 4 : 8;
+    if (std::is_same<R, float>::value) return N >= 1024 && MODE == INV ? 4 : 8;
     if (N >= 1024) return MODE == XMUL ? 2 : 4;
     if (std::is_same<R, double>::value) return N >= 128 ? 2 : 4;
     return N >= 512 && MODE != XMUL ? 8 : 4;
@@ -212,6 +213,14 @@ template <class R, int N, int LGB, class K = R> constexpr int line_threads()
 {
     return (N / PlanOf<K, N>::E) << (LGB >= 0 ? LGB : lg_max<R, N>());
 }
+// The runtime-tile kernel of 32-value plans is held at 128 registers (142 to 186 without a
+// cap), so that two CTAs of 256 threads share an SM.
+template <class R, int N, int LGB, class K = R> constexpr int line_min_blocks()
+{
+    constexpr int threads = line_threads<R, N, LGB, K>();
+    if (LGB < 0) return std::is_same<R, float>::value && PlanOf<K, N>::E >= 32 ? 65536 / (128 * threads) : 1;
+    return min_blocks<K, N, threads>();
+}
 template <int N> constexpr int lg_default() { return N >= 1024 ? 2 : 3; }
 
 // ------------------------------------------------------------------ asynchronous copies
@@ -219,6 +228,11 @@ SP_D void cp_async16(void* smem, const void* gmem)
 {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+SP_D void cp_async4(void* smem, const void* gmem)
+{
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
 }
 SP_D void cp_async8(void* smem, const void* gmem)
 {
@@ -232,7 +246,33 @@ SP_D void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "mem
 // multiplier values into shared memory with cp.async when its tile starts, so the loads
 // overlap the forward transform without holding registers; N B values of R per CTA.
 template <class R, int MODE> constexpr bool stage_m() { return MODE == XMUL && sizeof(R) >= 8; }
-template <class R, int N, int MODE> constexpr size_t stage_m_bytes(int B) { return stage_m<R, MODE>() ? sizeof(R) * (size_t)N * B : 0; }
+// FP32 at 20 values a thread or more copies the tile's multiplier rows (|kx| = 0 .. N/2) the
+// same way, by rows: half of the bytes of one value an output, and E registers fewer, which
+// with one exchange buffer and a cap of 128 registers doubles the warps an SM (8 to 16 at
+// 1024).  x passes, us, values in registers against rows: 512^3 3034 / 1957, 250^3 (F = 512)
+// 366 / 208, 300^3 (640) 986 / 723, 200^3 (400) 135 / 117, 150^3 (320) 87 / 72.  Twelve and
+// sixteen values a thread leave registers enough.
+template <class R, int N, int MODE, class K = R> constexpr bool row_m()
+{
+    return MODE == XMUL && std::is_same<R, float>::value && PlanOf<K, N>::E >= 20;
+}
+template <class R, int N, int MODE, class K = R> SP_HD constexpr size_t stage_m_bytes(int B)
+{
+    if (row_m<R, N, MODE, K>()) return (sizeof(R) * (size_t)(N / 2 + 1) * B + 15) / 16 * 16;
+    return stage_m<R, MODE>() ? sizeof(R) * (size_t)N * B : 0;
+}
+// Exchange buffers of a CTA of B columns (staged rows: two where four CTAs still fit an SM).
+template <class R, int N, int MODE, class K = R> SP_HD constexpr bool line_two_buffers(int B)
+{
+    const size_t buf = sizeof(cpx<R>) * strided_size<R, K, N>(B);
+    if (row_m<R, N, MODE, K>()) return 2 * buf + stage_m_bytes<R, N, MODE, K>(B) <= 56 * 1024;
+    return two_buffers(buf, pass_tw_bytes<R, N, K>());
+}
+template <class R, int N, int MODE, class K = R> SP_HD constexpr size_t line_smem(int B)
+{
+    return pass_tw_bytes<R, N, K>() + (line_two_buffers<R, N, MODE, K>(B) ? 2 : 1) * sizeof(cpx<R>) * strided_size<R, K, N>(B) +
+           stage_m_bytes<R, N, MODE, K>(B);
+}
 
 // One tile of a line pass: B columns (c = cb B + b) of outer index o, right-hand side
 // `batch`; all threads of the block take part.  `smraw` is the pass's dynamic shared
@@ -246,7 +286,7 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
     constexpr int R0 = PlanOf<K, N>::R[0];
     const int lgB = LGB >= 0 ? LGB : a.lgB, B = 1 << lgB;
     const int BUF = strided_size<R, K, N>(B);
-    const bool DB = two_buffers(sizeof(cpx<R>) * BUF, pass_tw_bytes<R, N, K>());
+    const bool DB = line_two_buffers<R, N, MODE, K>(B);
     cpx<R>* tws_s = reinterpret_cast<cpx<R>*>(smraw);
     cpx<R>* sm0 = tws_s + pass_tw_bytes<R, N, K>() / sizeof(cpx<R>);
     cpx<R>* sm1 = DB ? sm0 + BUF : sm0;
@@ -280,14 +320,26 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
     // x pass: the multiplier values of this thread's outputs are fetched before the forward
     // transform, so their latency overlaps its arithmetic: into registers for FP32, into
     // shared memory by cp.async for the 8-byte types (whose registers hold the transform)
-    constexpr bool PREFETCH_M = MODE == XMUL && sizeof(R) == 4;
+    constexpr bool ROW_M = row_m<R, N, MODE, K>();
+    constexpr bool PREFETCH_M = MODE == XMUL && sizeof(R) == 4 && !ROW_M;
     constexpr bool STAGE_M = stage_m<R, MODE>();
     R mv[MODE == XMUL ? E : 1];
     const R* M = static_cast<const R*>(a.M);
     const int ko = o <= a.No / 2 ? o : a.No - o;
     const long long mrow = (long long)ko * (a.nh_line + 1);
-    R* mst = reinterpret_cast<R*>(sm1 + BUF);  // STAGE_M: [j][thread]
-    if constexpr (PREFETCH_M) {
+    R* mst = reinterpret_cast<R*>(sm1 + BUF);  // STAGE_M: [j][thread]; ROW_M: [|kx|][column]
+    if constexpr (ROW_M) {
+        const R* src = M + mrow * a.ldzM + (long long)cb * B;
+        if (B >= 4 && ((uintptr_t)M & 15) == 0 && (a.ldzM & 3) == 0 && cb * B + B <= a.ldzM) {
+            const int lgc = lgB - 2;  // log2 of the 16-byte chunks of a row
+            for (int q = tid; q < (N / 2 + 1) << lgc; q += blockDim.x)
+                cp_async16(mst + 4 * q, src + (long long)(q >> lgc) * a.ldzM + 4 * (q & ((1 << lgc) - 1)));
+        } else {
+            for (int q = tid; q < (N / 2 + 1) << lgB; q += blockDim.x)
+                if (cb * B + (q & (B - 1)) < a.ncol) cp_async4(mst + q, src + (long long)(q >> lgB) * a.ldzM + (q & (B - 1)));
+        }
+        cp_async_commit();
+    } else if constexpr (PREFETCH_M) {
 #pragma unroll
         for (int j = 0; j < E; ++j) {
             const int e = last_element<K, N, false>(t, j);
@@ -307,6 +359,9 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
     }
     __syncthreads();
     cpx<R>* fresh;
+    // the copies were issued with the tile's loads and land with them; the exchange barriers
+    // of the forward transform make every thread's visible to all
+    if constexpr (ROW_M) cp_async_wait_all();
     if constexpr (MODE == INV) {
         fresh = run_stages<R, N, true, +1, false, K>(v, sm0, sm1, layi, tws, t);
     } else {
@@ -318,6 +373,9 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
         for (int j = 0; j < E; ++j) {
             if constexpr (STAGE_M) {
                 mv[j] = cv ? mst[j * blockDim.x + tid] : Num<R>::c(0.0);
+            } else if constexpr (ROW_M) {
+                const int e = last_element<K, N, false>(t, j);
+                mv[j] = cv ? mst[((e <= N / 2 ? e : N - e) << lgB) + b] : Num<R>::c(0.0);
             } else if constexpr (!PREFETCH_M) {
                 const int e = last_element<K, N, false>(t, j);
                 const int ke = e <= N / 2 ? e : N - e;
@@ -340,7 +398,7 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
 }
 
 template <class R, int N, int MODE, int LGB, class K = R>
-__global__ void __launch_bounds__(line_threads<R, N, LGB, K>(), LGB >= 0 ? min_blocks<K, N, line_threads<R, N, LGB, K>()>() : 1)
+__global__ void __launch_bounds__(line_threads<R, N, LGB, K>(), line_min_blocks<R, N, LGB, K>())
     k2_line(LArgs a)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -734,9 +792,7 @@ sp_status launch_line(const LArgs& a, int outer, int batch, cudaStream_t st)
     if (B < 1 || B > lanes_b_max<R, N>() || (B & (B - 1))) return sp_fail(SP_ERR_INVALID, "bad line tile %d", B);
     ab.lgB = 0;
     while ((1 << ab.lgB) < B) ++ab.lgB;
-    const size_t buf = sizeof(cpx<R>) * strided_size<R, K, N>(B);
-    const size_t twb = pass_tw_bytes<R, N, K>();
-    const size_t smem = twb + (two_buffers(buf, twb) ? 2 : 1) * buf + stage_m_bytes<R, N, MODE>(B);
+    const size_t smem = line_smem<R, N, MODE, K>(B);
     dim3 grid((unsigned)((a.ncol + B - 1) / B), (unsigned)outer, (unsigned)batch);
     sp_status rc;
     constexpr size_t psmem = pipe_smem<R, N, MODE, K>();
@@ -1125,9 +1181,7 @@ template <class R, int N> constexpr bool persist_ok()
 template <class R, int N> constexpr size_t persist_smem()
 {
     constexpr int B = 1 << persist_lgb<R, N>();
-    constexpr size_t lbuf = sizeof(cpx<R>) * (size_t)strided_size<R, R, N>(B);
-    constexpr size_t ltw = pass_tw_bytes<R, N>();
-    constexpr size_t line = ltw + (two_buffers(lbuf, ltw) ? 2 : 1) * lbuf + stage_m_bytes<R, N, XMUL>(B);
+    constexpr size_t fl = line_smem<R, N, FWD>(B), xl = line_smem<R, N, XMUL>(B), line = fl > xl ? fl : xl;
     constexpr size_t zbuf = sizeof(cpx<R>) * (size_t)persist_bz<R, N>() * line_ld<ZKey<R>, N>();
     constexpr size_t ztw = pass_tw_bytes<R, N, ZKey<R>>();
     constexpr size_t zs = ztw + (two_buffers(zbuf, ztw) ? 2 : 1) * zbuf;
