@@ -20,12 +20,14 @@ namespace v2 {
 // Largest tile (columns) and the register cap, as resident CTAs of that size: 16-byte types
 // run E = 12 and above at 168 registers (spilling below it costs 10 to 40 %; 128 where a
 // line has 64 threads or more), fewer values at 128 (96 for E = 6); 8-byte types at 64, 96
-// or 128 by E.
+// or 128 by E.  CTAs of 8-byte types go up to 512 threads, so that lines of 33 to 64 threads
+// keep tiles of 8 columns, 64 contiguous bytes a row (x / y forward / y inverse, us, 4 columns
+// against 8: 210^3 (F = 432) 224/72/80 / 177/59/67, 285^3 (576) 558/166/191 / 446/142/172).
 template <class R, class K, int N> constexpr int rag_b_max()
 {
     constexpr int T = N / PlanOf<K, N>::E;
     int b = 16;
-    while (b > 2 && b * T > 256) b /= 2;
+    while (b > 2 && b * T > (sizeof(cpx<R>) >= 16 ? 256 : 512)) b /= 2;
     return b;
 }
 template <class R, class K, int N> constexpr int rag_min_blocks(int threads)
@@ -90,10 +92,34 @@ inline int rag_pairs(int T, int bmax, long long pairs)
     return best;
 }
 
+// FP32 y passes that run the pipelined kernel (k3_line): they move a row in and half a row out,
+// or the reverse, with one transform between, so what bounds them is the latency of the loads,
+// which the pipeline takes out.  Inverse passes load whole rows and gain from F = 256 up
+// (us, plain tile against pipeline: 125^3 16.4 / 13.8, 200^3 66 / 41, 250^3 144 / 74, 285^3
+// 172 / 144), forward passes, whose loads are half as many, from 400 (200^3 47 / 41, 250^3
+// 102 / 72; 240x180x75 24.8 / 26.7).  Few tiles leave the persistent CTAs without a next one to
+// load (39x172x122, 1326 tiles, three a CTA: 3 % slower; 240x180x75, 2640: 2 % faster): from 16
+// an SM.  Eight values a thread have warps enough without it, and the x pass computes twice as
+// long a byte (200^3 117 / 144).
+constexpr long long kPipeTiles = 16 * 152;
+template <class R, int N, int MODE> constexpr bool rag_pipe()
+{
+    return std::is_same<R, float>::value && PlanOf<R, N>::E >= 12 &&
+           N <= 864 &&
+           (MODE == INV ? N >= 256 : MODE == FWD && N >= 400) && pipe_smem<R, N, MODE, R, true>() <= 110 * 1024;
+}
 template <class R, int N, int MODE> sp_status rag_line(const LArgs& a, int outer, int batch, cudaStream_t st)
 {
     constexpr int T = N / PlanOf<R, N>::E;
     LArgs ab = a;
+    if constexpr (rag_pipe<R, N, MODE>()) {
+        constexpr int B = 1 << lg_default<N>();
+        if ((long long)((a.ncol + B - 1) / B) * outer * batch >= kPipeTiles && pipe_fits<R, N, MODE, R, true>(a)) {
+            ab.B = B;
+            ab.lgB = lg_default<N>();
+            return launch_pipe<R, N, MODE, R, true>(ab, outer, batch, st);
+        }
+    }
     ab.B = rag_tile<R, N>(T, rag_b_max<R, R, N>(), a.ncol, (long long)outer * batch);
     ab.lgB = 0;
     while ((1 << ab.lgB) < ab.B) ++ab.lgB;

@@ -246,15 +246,14 @@ SP_D void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "mem
 // multiplier values into shared memory with cp.async when its tile starts, so the loads
 // overlap the forward transform without holding registers; N B values of R per CTA.
 template <class R, int MODE> constexpr bool stage_m() { return MODE == XMUL && sizeof(R) >= 8; }
-// FP32 at 20 values a thread or more copies the tile's multiplier rows (|kx| = 0 .. N/2) the
+// FP32 at 12 values a thread or more copies the tile's multiplier rows (|kx| = 0 .. N/2) the
 // same way, by rows: half of the bytes of one value an output, and E registers fewer, which
 // with one exchange buffer and a cap of 128 registers doubles the warps an SM (8 to 16 at
 // 1024).  x passes, us, values in registers against rows: 512^3 3034 / 1957, 250^3 (F = 512)
-// 366 / 208, 300^3 (640) 986 / 723, 200^3 (400) 135 / 117, 150^3 (320) 87 / 72.  Twelve and
-// sixteen values a thread leave registers enough.
+// 366 / 208, 200^3 (400) 135 / 117, 150^3 (320) 87 / 72, 125^3 (256) 37 / 31.
 template <class R, int N, int MODE, class K = R> constexpr bool row_m()
 {
-    return MODE == XMUL && std::is_same<R, float>::value && PlanOf<K, N>::E >= 20;
+    return MODE == XMUL && std::is_same<R, float>::value && PlanOf<K, N>::E >= 12;
 }
 template <class R, int N, int MODE, class K = R> SP_HD constexpr size_t stage_m_bytes(int B)
 {
@@ -411,7 +410,8 @@ __global__ void __launch_bounds__(line_threads<R, N, LGB, K>(), line_min_blocks<
 // index, column block) with a stride of gridDim.x.  A tile's input rows (B contiguous
 // complex values each) are copied into a shared-memory stage with cp.async; after the
 // threads have moved the current tile's values from the stage into registers, the copies
-// of the next tile are issued, so they land while the current tile computes.
+// of the next tile are issued, so they land while the current tile computes.  RAG: as in
+// line_tile; only the axis's a.nlim rows are copied.
 
 struct PArgs {
     LArgs a;
@@ -422,7 +422,8 @@ struct PArgs {
 
 template <class R, int N, int MODE> constexpr int stage_rows() { return MODE == INV ? N : N / 2; }
 // Two exchange buffers when they fit beside the twiddles and the stage in 110 KB (two CTAs
-// per SM), else one.
+// per SM), else one.  On ragged lines 75 KB (three CTAs; y forward/inverse, us, at 110 KB
+// against 75: 210^3 59/78 / 61/68, 200^3 41/47 / 41/41).
 // The y passes of the 32-value plan at 512 (one exchange a transform) trade the second
 // buffer for a third resident CTA (measured: y passes 10 % faster; the 1024 passes are
 // faster with two buffers and two CTAs).  So does the FP32 x pass of that plan, whose
@@ -443,24 +444,24 @@ template <class R, int N, int MODE, class K = R> constexpr size_t pipe_mstage_by
 {
     return pipe_mstage<R, N, MODE, K>() ? sizeof(R) * (size_t)(N / 2 + 1) * (1 << lg_default<N>()) : 0;
 }
-template <class R, int N, int MODE, class K = R> constexpr bool pipe_two_buffers()
+template <class R, int N, int MODE, class K = R, bool RAG = false> constexpr bool pipe_two_buffers()
 {
     constexpr int B = 1 << lg_default<N>();
     constexpr size_t buf = sizeof(cpx<R>) * (size_t)strided_size<R, K, N>(B);
     constexpr size_t twb = sizeof(cpx<R>) * tw_entries<K, N>();
     return !pipe_third_cta<R, N, MODE, K>() &&
-           twb + 2 * buf + sizeof(cpx<R>) * (size_t)stage_rows<R, N, MODE>() * B <= 110 * 1024;
+           twb + 2 * buf + sizeof(cpx<R>) * (size_t)stage_rows<R, N, MODE>() * B <= (RAG ? 75 : 110) * 1024;
 }
-template <class R, int N, int MODE, class K = R> constexpr size_t pipe_smem()
+template <class R, int N, int MODE, class K = R, bool RAG = false> constexpr size_t pipe_smem()
 {
     constexpr int B = 1 << lg_default<N>();
     constexpr size_t buf = sizeof(cpx<R>) * (size_t)strided_size<R, K, N>(B);
     constexpr size_t twb = sizeof(cpx<R>) * tw_entries<K, N>();
-    return twb + (pipe_two_buffers<R, N, MODE, K>() ? 2 : 1) * buf + sizeof(cpx<R>) * (size_t)stage_rows<R, N, MODE>() * B +
+    return twb + (pipe_two_buffers<R, N, MODE, K, RAG>() ? 2 : 1) * buf + sizeof(cpx<R>) * (size_t)stage_rows<R, N, MODE>() * B +
            pipe_mstage_bytes<R, N, MODE, K>();
 }
 
-template <class R, int N, int MODE, class K = R>
+template <class R, int N, int MODE, class K = R, bool RAG = false>
 __global__ void __launch_bounds__(line_threads<R, N, lg_default<N>(), K>(),
                                   pipe_third_cta<R, N, MODE, K>() ? 3 : min_blocks<K, N, line_threads<R, N, lg_default<N>(), K>()>())
     k3_line(PArgs pa)
@@ -481,7 +482,7 @@ __global__ void __launch_bounds__(line_threads<R, N, lg_default<N>(), K>(),
     grid_dependency();
     const LArgs& a = pa.a;
     const int BUF = strided_size<R, K, N>(B);
-    constexpr bool DB = pipe_two_buffers<R, N, MODE, K>();
+    constexpr bool DB = pipe_two_buffers<R, N, MODE, K, RAG>();
     extern __shared__ __align__(16) unsigned char smraw[];
     cpx<R>* tws = reinterpret_cast<cpx<R>*>(smraw);
     cpx<R>* sm0 = tws + tw_entries<K, N>();
@@ -515,7 +516,8 @@ __global__ void __launch_bounds__(line_threads<R, N, lg_default<N>(), K>(),
         const int xo = a.reverse ? pa.outer - 1 - x.o : x.o;
         const char* src = reinterpret_cast<const char*>(static_cast<const cpx<R>*>(a.in) + x.batch * a.in_bs +
                                                         xo * a.in_os + x.cb * B);
-        for (int q = tid; q < NIN * CH; q += blockDim.x) {
+        const int rows = RAG && MODE != INV ? a.nlim : NIN;
+        for (int q = tid; q < rows * CH; q += blockDim.x) {
             const int row = q / CH, ch = q % CH;
             cp_async16(reinterpret_cast<char*>(stg) + (size_t)row * B * sizeof(cpx<R>) + ch * 16,
                        src + (long long)row * a.in_es * (long long)sizeof(cpx<R>) + ch * 16);
@@ -556,7 +558,9 @@ __global__ void __launch_bounds__(line_threads<R, N, lg_default<N>(), K>(),
         } else {
 #pragma unroll
             for (int j = 0; j < E; ++j)
-                v[j] = ((j % R0) < R0 / 2) ? stg[first_element<K, N, false>(t, j) * B + b] : czero<R>();
+                v[j] = ((j % R0) < R0 / 2 && (!RAG || first_element<K, N, false>(t, j) < a.nlim))
+                           ? stg[first_element<K, N, false>(t, j) * B + b]
+                           : czero<R>();
         }
         constexpr bool PREFETCH_M = MODE == XMUL && sizeof(R) == 4 && !MST;
         R mv[MODE == XMUL ? E : 1];
@@ -610,7 +614,8 @@ __global__ void __launch_bounds__(line_threads<R, N, lg_default<N>(), K>(),
         } else {
 #pragma unroll
             for (int j = 0; j < E; ++j)
-                if ((j % R0) < R0 / 2 && cv) out[last_element<K, N, true>(t, j) * a.out_es] = norm(v[j]);
+                if ((j % R0) < R0 / 2 && cv && (!RAG || last_element<K, N, true>(t, j) < a.nlim))
+                    out[last_element<K, N, true>(t, j) * a.out_es] = norm(v[j]);
         }
         __syncthreads();  // exchange buffers free before the next tile's first write
         cur = nxt;
@@ -782,6 +787,44 @@ template <auto KERNEL> inline sp_status smem_attr(size_t bytes)
     return rc;
 }
 
+// The pipelined persistent kernel takes the default tile, inputs whose rows are 16-byte
+// aligned (the workspace), and a stage that still leaves two CTAs per SM; the staged
+// multiplier rows are copied in 16-byte chunks as well.
+template <class R, int N, int MODE, class K = R, bool RAG = false> bool pipe_fits(const LArgs& a)
+{
+    constexpr int B = 1 << lg_default<N>();
+    const bool rows_aligned = ((uintptr_t)a.in % 16 == 0) && (a.in_es * sizeof(cpx<R>)) % 16 == 0 &&
+                              (a.in_os * sizeof(cpx<R>)) % 16 == 0 && (a.in_bs * sizeof(cpx<R>)) % 16 == 0;
+    const bool m_aligned = !pipe_mstage<R, N, MODE, K>() ||
+                           ((uintptr_t)a.M % 16 == 0 && (a.ldzM * sizeof(R)) % 16 == 0 && (a.ncol + B - 1) / B * B <= a.ldzM);
+    return pipe_smem<R, N, MODE, K, RAG>() <= 110 * 1024 && rows_aligned && m_aligned && (a.ncol + B - 1) / B * B <= a.in_ld;
+}
+template <class R, int N, int MODE, class K = R, bool RAG = false>
+sp_status launch_pipe(const LArgs& a, int outer, int batch, cudaStream_t st)
+{
+    constexpr int B = 1 << lg_default<N>(), threads = N / PlanOf<K, N>::E * B;
+    constexpr size_t smem = pipe_smem<R, N, MODE, K, RAG>();
+    sp_status rc;
+    if ((rc = smem_attr<k3_line<R, N, MODE, K, RAG>>(smem))) return rc;
+    static std::atomic<int> per_sm_cached{0};  // resident CTAs per SM (same on every GB300)
+    int per_sm = per_sm_cached.load(std::memory_order_relaxed);
+    if (!per_sm) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k3_line<R, N, MODE, K, RAG>, threads, smem);
+        if (per_sm < 1) per_sm = 1;
+        per_sm_cached.store(per_sm, std::memory_order_relaxed);
+    }
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    PArgs pa;
+    pa.a = a;
+    pa.outer = outer;
+    pa.ncb = (a.ncol + B - 1) / B;
+    pa.ntiles = batch * outer * pa.ncb;
+    const int nblocks = pa.ntiles < per_sm * sms ? pa.ntiles : per_sm * sms;
+    return launch_pass(k3_line<R, N, MODE, K, RAG>, dim3(nblocks), threads, smem, st, pa, a.dependent != 0, "v2 line pass");
+}
+
 template <class R, int N, int MODE, class K = R>
 sp_status launch_line(const LArgs& a, int outer, int batch, cudaStream_t st)
 {
@@ -795,34 +838,8 @@ sp_status launch_line(const LArgs& a, int outer, int batch, cudaStream_t st)
     const size_t smem = line_smem<R, N, MODE, K>(B);
     dim3 grid((unsigned)((a.ncol + B - 1) / B), (unsigned)outer, (unsigned)batch);
     sp_status rc;
-    constexpr size_t psmem = pipe_smem<R, N, MODE, K>();
-    // pipelined persistent kernel: default tile, inputs whose rows are 16-byte aligned
-    // (the workspace), and a stage that still leaves two CTAs per SM
-    const bool rows_aligned = ((uintptr_t)a.in % 16 == 0) && (a.in_es * sizeof(cpx<R>)) % 16 == 0 &&
-                              (a.in_os * sizeof(cpx<R>)) % 16 == 0 && (a.in_bs * sizeof(cpx<R>)) % 16 == 0;
-    // the staged multiplier rows are copied in 16-byte chunks as well
-    const bool m_aligned = !pipe_mstage<R, N, MODE, K>() ||
-                           ((uintptr_t)a.M % 16 == 0 && (a.ldzM * sizeof(R)) % 16 == 0 && (a.ncol + B - 1) / B * B <= a.ldzM);
-    if (ab.lgB == lg_default<N>() && psmem <= 110 * 1024 && rows_aligned && m_aligned &&
-        (a.ncol + B - 1) / B * B <= a.in_ld) {
-        if ((rc = smem_attr<k3_line<R, N, MODE, K>>(psmem))) return rc;
-        static std::atomic<int> per_sm_cached{0};  // resident CTAs per SM (same on every GB300)
-        int per_sm = per_sm_cached.load(std::memory_order_relaxed);
-        if (!per_sm) {
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k3_line<R, N, MODE, K>, (N / E) * B, psmem);
-            if (per_sm < 1) per_sm = 1;
-            per_sm_cached.store(per_sm, std::memory_order_relaxed);
-        }
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        PArgs pa;
-        pa.a = ab;
-        pa.outer = outer;
-        pa.ncb = (a.ncol + B - 1) / B;
-        pa.ntiles = batch * outer * pa.ncb;
-        const int nblocks = pa.ntiles < per_sm * sms ? pa.ntiles : per_sm * sms;
-        return launch_pass(k3_line<R, N, MODE, K>, dim3(nblocks), (N / E) * B, psmem, st, pa, a.dependent != 0, "v2 line pass");
+    if (ab.lgB == lg_default<N>() && pipe_fits<R, N, MODE, K>(ab)) {
+        return launch_pipe<R, N, MODE, K>(ab, outer, batch, st);
     } else if (ab.lgB == lg_default<N>()) {
         if ((rc = smem_attr<k2_line<R, N, MODE, lg_default<N>(), K>>(smem))) return rc;
         return launch_pass(k2_line<R, N, MODE, lg_default<N>(), K>, grid, (N / E) * B, smem, st, ab, a.dependent != 0, "v2 line pass");
