@@ -10,7 +10,7 @@
 //
 // The kernels are those of sp_v2.cuh with a bound on the line's grid points (RAG): rows at
 // and above n are zero on input and not written on output.  Measured at n = 101 (double-
-// float): see the design doc's table; the runtime-radix passes of sp_passes.cu took 1.17 ms.
+// float): 171 us; the runtime-radix passes of sp_passes.cu took 1.17 ms.
 #pragma once
 
 #include "sp_v2.cuh"
@@ -23,24 +23,32 @@ namespace v2 {
 // or 128 by E.  CTAs of 8-byte types go up to 512 threads, so that lines of 33 to 64 threads
 // keep tiles of 8 columns, 64 contiguous bytes a row (x / y forward / y inverse, us, 4 columns
 // against 8: 210^3 (F = 432) 224/72/80 / 177/59/67, 285^3 (576) 558/166/191 / 446/142/172).
-template <class R, class K, int N> constexpr int rag_b_max()
+// Double-float passes of one transform on eight values and 32 threads or more a line are light:
+// 96 registers hold them (y forward/inverse, z forward/inverse, us, 128 against 96: 150^3 70/73,
+// 59/54 / 66/68, 55/49; 300^3 599/639, 401/401 / 587/578, 346/345 with tiles of 4 columns on 320
+// threads; the x pass spills and loses 5 to 10 %).
+template <class R, class K, int N, int MODE> constexpr bool rag_light()
 {
-    constexpr int T = N / PlanOf<K, N>::E;
-    int b = 16;
-    while (b > 2 && b * T > (sizeof(cpx<R>) >= 16 ? 256 : 512)) b /= 2;
+    return std::is_same<R, df32>::value && PlanOf<K, N>::E <= 8 && N / PlanOf<K, N>::E >= 32 && MODE != XMUL;
+}
+template <class R, int N, int MODE> constexpr int rag_b_max()
+{
+    constexpr int T = N / PlanOf<R, N>::E;
+    int b = sizeof(cpx<R>) >= 16 && T >= 32 ? 4 : 16;  // the most that rag_tile takes
+    while (b > 2 && b * T > (sizeof(cpx<R>) < 16 ? 512 : (rag_light<R, R, N, MODE>() ? 320 : 256))) b /= 2;
     return b;
 }
-template <class R, class K, int N> constexpr int rag_min_blocks(int threads)
+template <class R, class K, int N, int MODE> constexpr int rag_min_blocks(int threads)
 {
     constexpr int E = PlanOf<K, N>::E, T = N / E;
-    constexpr int cap = sizeof(cpx<R>) >= 16 ? (E <= 6 ? 96 : (E >= 12 && T < 64 ? 168 : 128)) : (E <= 8 ? 64 : (E <= 16 ? 96 : 128));
+    constexpr int cap = sizeof(cpx<R>) >= 16 ? (E <= 6 || rag_light<R, K, N, MODE>() ? 96 : (E >= 12 && T < 64 ? 168 : 128)) : (E <= 8 ? 64 : (E <= 16 ? 96 : 128));
     const int b = 65536 / (cap * threads);
     return b < 1 ? 1 : b;
 }
 
 template <class R, int N, int MODE>
-__global__ void __launch_bounds__((N / PlanOf<R, N>::E) * rag_b_max<R, R, N>(),
-                                  rag_min_blocks<R, R, N>((N / PlanOf<R, N>::E) * rag_b_max<R, R, N>())) k_rag_line(LArgs a)
+__global__ void __launch_bounds__((N / PlanOf<R, N>::E) * rag_b_max<R, N, MODE>(),
+                                  rag_min_blocks<R, R, N, MODE>((N / PlanOf<R, N>::E) * rag_b_max<R, N, MODE>())) k_rag_line(LArgs a)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     grid_dependency();
@@ -54,7 +62,7 @@ template <class R, int N> constexpr int rag_pairs_max()
 }
 template <class R, class Tio, int N, bool FORWARD>
 __global__ void __launch_bounds__((N / PlanOf<ZKey<R>, N>::E) * rag_pairs_max<R, N>(),
-                                  rag_min_blocks<R, ZKey<R>, N>((N / PlanOf<ZKey<R>, N>::E) * rag_pairs_max<R, N>()))
+                                  rag_min_blocks<R, ZKey<R>, N, FWD>((N / PlanOf<ZKey<R>, N>::E) * rag_pairs_max<R, N>()))
     k_rag_z(ZArgs2 a)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -120,7 +128,7 @@ template <class R, int N, int MODE> sp_status rag_line(const LArgs& a, int outer
             return launch_pipe<R, N, MODE, R, true>(ab, outer, batch, st);
         }
     }
-    ab.B = rag_tile<R, N>(T, rag_b_max<R, R, N>(), a.ncol, (long long)outer * batch);
+    ab.B = rag_tile<R, N>(T, rag_b_max<R, N, MODE>(), a.ncol, (long long)outer * batch);
     ab.lgB = 0;
     while ((1 << ab.lgB) < ab.B) ++ab.lgB;
     const size_t smem = line_smem<R, N, MODE>(ab.B);

@@ -134,6 +134,13 @@ template <> struct PlanOf<float, 128> : Plan128Radix16 {};
 // register caps: 16-byte values want 8 to 12 values a thread (double-float at 200: 82 us
 // with 10-10-2 and E = 10, 104 us with 20-10 and E = 20), FP32 wants fewer stages (at 400:
 // 20-20 and E = 20, 4.6 ps a point, against 5.8 with 10-10-4).
+// Lengths 5 x 2^k and 400 would need 20 values a thread, or a fourth stage, for their factors 5
+// to divide E.  Their middle stage instead gives some threads a butterfly fewer (one in five
+// idles for a third of the transform), on 8 or 10 values: whole solves, us, double-float 77^3
+// (F = 160) 101 / 85, 150^3 (320) 636 / 521, 200^3 (400) 1458 / 1220, 300^3 (640) 7050 / 4447;
+// FP64 200^3 6663 / 6210, 310^3 26390 / 24780, but 150^3 2787 / 2909 and 77^3 383 / 401 (its pipe
+// is full either way: FP64 keeps the 20-point plans at 160 and 320); FP32 77^3 40 / 36, 300^3
+// 1617 / 1281, and at 320 and 400 the z passes only (155^3 22/29 / 21/20, x 72 / 91).
 template <> struct FFTPlan<16> : PlanE<4, 4, 4> {};
 template <> struct FFTPlan<32> : PlanE<8, 8, 4> {};
 template <> struct FFTPlan<48> : PlanE<12, 12, 4> {};
@@ -141,34 +148,37 @@ template <> struct FFTPlan<72> : PlanE<12, 12, 6> {};
 template <> struct FFTPlan<80> : PlanE<20, 20, 4> {};
 template <> struct FFTPlan<96> : PlanE<12, 6, 4, 4> {};
 template <> struct FFTPlan<144> : PlanE<12, 12, 12> {};
-template <> struct FFTPlan<160> : PlanE<20, 20, 4, 2> {};
+template <> struct FFTPlan<160> : PlanE<8, 8, 5, 4> {};
 template <> struct FFTPlan<200> : PlanE<10, 10, 10, 2> {};
 template <> struct FFTPlan<216> : PlanE<6, 6, 6, 6> {};
 template <> struct FFTPlan<288> : PlanE<12, 12, 6, 4> {};
-template <> struct FFTPlan<320> : PlanE<20, 20, 4, 4> {};
-template <> struct FFTPlan<400> : PlanE<10, 10, 10, 2, 2> {};
+template <> struct FFTPlan<320> : PlanE<8, 8, 5, 8> {};
+template <> struct FFTPlan<400> : PlanE<10, 10, 4, 10> {};
 template <> struct FFTPlan<432> : PlanE<12, 12, 6, 6> {};
 template <> struct FFTPlan<576> : PlanE<12, 12, 12, 4> {};
-template <> struct FFTPlan<640> : PlanE<20, 20, 2, 4, 4> {};
+template <> struct FFTPlan<640> : PlanE<8, 8, 10, 8> {};
 template <> struct FFTPlan<768> : PlanE<12, 4, 4, 4, 12> {};
 template <> struct FFTPlan<864> : PlanE<12, 12, 12, 6> {};
 template <> struct FFTPlan<1280> : PlanE<20, 20, 4, 4, 4> {};
 template <> struct FFTPlan<1536> : PlanE<12, 12, 4, 4, 4, 2> {};
 template <> struct FFTPlan<2048> : PlanE<16, 16, 16, 8> {};
 template <> struct PlanOf<float, 96> : PlanE<24, 12, 8> {};
-template <> struct PlanOf<float, 160> : PlanE<20, 10, 4, 4> {};
 template <> struct PlanOf<float, 200> : PlanE<20, 20, 10> {};
 template <> struct PlanOf<float, 400> : PlanE<20, 20, 20> {};
-template <> struct PlanOf<float, 640> : PlanE<20, 4, 4, 4, 10> {};
+template <> struct PlanOf<float, 320> : PlanE<20, 20, 4, 4> {};
+template <> struct PlanOf<double, 160> : PlanE<20, 20, 4, 2> {};
+template <> struct PlanOf<double, 320> : PlanE<20, 20, 4, 4> {};
 template <> struct PlanOf<float, 768> : PlanE<24, 8, 8, 12> {};
 
 // Plan key of the z passes (contiguous real lines, packed in pairs): the type's own plan,
 // except FP32 at 512 and 1024, whose z passes run faster on 8-8-8 and 16-8-8 than on the
-// radix-32 plans of its line passes.  Each axis has its own staged twiddle table, so the
-// z axis can differ.
+// radix-32 plans of its line passes, and at 320 and 400 (above).  Each axis has its own staged
+// twiddle table, so the z axis can differ.
 template <class R> struct ZKey {};
 template <class R, int N> struct PlanOf<ZKey<R>, N> : PlanOf<R, N> {};
 template <> struct PlanOf<ZKey<float>, 512> : FFTPlan<512> {};
+template <> struct PlanOf<ZKey<float>, 320> : FFTPlan<320> {};
+template <> struct PlanOf<ZKey<float>, 400> : FFTPlan<400> {};
 template <> struct PlanOf<ZKey<float>, 1024> : Plan1024Radix16 {};
 
 // Alternative radix plans of the line passes, which the autotuner times against the
@@ -556,17 +566,19 @@ SP_D void fill_stage_twiddles(cpx<R>* tws, const cpx<R>* __restrict__ tw, int ti
     }
 }
 
-// A plan is usable when its radices multiply to N and every radix divides E (each thread
-// runs whole butterflies).
+// A plan is usable when its radices multiply to N and the first and the last divide E (each
+// thread enters and leaves with E values of whole butterflies).  A middle radix may leave
+// butterflies over: threads take up to ceil((N / RAD) / T) of them, in the last round only the
+// first threads of the line.
 template <class K, int N> constexpr bool plan_ok()
 {
     int prod = 1;
     for (int i = 0; i < PlanOf<K, N>::NS; ++i) {
         const int r = PlanOf<K, N>::R[i];
-        if (PlanOf<K, N>::E % r != 0) return false;
+        if ((i == 0 || i + 1 == PlanOf<K, N>::NS) && PlanOf<K, N>::E % r != 0) return false;
         prod *= r;
     }
-    return prod == N;
+    return prod == N && N % PlanOf<K, N>::E == 0;
 }
 
 template <class Lay> constexpr bool steps(int d) { return Lay::per == 0 || d % (Lay::per == 0 ? 1 : Lay::per) == 0; }
@@ -577,14 +589,17 @@ template <class R, int N, bool INV, int ST, class K = R> struct Stage {
     static constexpr int T = N / E;
     static constexpr int RAD = radix_at<K, N, INV>(ST);
     static constexpr int P = span_at<K, N, INV>(ST);
-    static constexpr int NB = E / RAD;
-    static constexpr int STRIDE = N / RAD;
+    static constexpr int STRIDE = N / RAD;           // butterflies of a line
+    static constexpr int NB = (STRIDE + T - 1) / T;  // of a thread, at most
+    static constexpr int EL = NB * RAD;              // values a thread holds in this stage
+    SP_D static bool has(int m, int t) { return T * (m + 1) <= STRIDE || t + T * m < STRIDE; }
 
     // inputs of this stage from shared memory: v[m RAD + r] = x[t + T m + r N/RAD]
-    template <class Lay> SP_D static void load(cpx<R> (&v)[E], const cpx<R>* sm, const Lay& lay, int t)
+    template <class Lay> SP_D static void load(cpx<R> (&v)[EL], const cpx<R>* sm, const Lay& lay, int t)
     {
 #pragma unroll
         for (int m = 0; m < NB; ++m) {
+            if (!has(m, t)) continue;
             if constexpr (steps<Lay>(STRIDE)) {
                 const cpx<R>* p0 = sm + lay(t + T * m);
                 const int st = lay.step(STRIDE);
@@ -598,10 +613,11 @@ template <class R, int N, bool INV, int ST, class K = R> struct Stage {
     }
 
     // twiddles and butterflies (S = -1 forward, +1 inverse); HALF: inputs r >= RAD/2 are zero
-    template <int S, bool HALF> SP_D static void compute(cpx<R> (&v)[E], const cpx<R>* tws, int t)
+    template <int S, bool HALF> SP_D static void compute(cpx<R> (&v)[EL], const cpx<R>* tws, int t)
     {
 #pragma unroll
         for (int m = 0; m < NB; ++m) {
+            if (!has(m, t)) continue;
             if constexpr (P > 1) {
                 const int k = (t + T * m) % P;
                 const cpx<R>* w = tws + tw_base<K, N, INV>() + tw_stage_offset<K, N, INV>(ST) + k * (RAD + 1);
@@ -630,10 +646,11 @@ template <class R, int N, bool INV, int ST, class K = R> struct Stage {
     }
 
     // outputs of this stage to shared memory: y[(i - k) RAD + k + q P] = v[m RAD + q]
-    template <class Lay> SP_D static void store(const cpx<R> (&v)[E], cpx<R>* sm, const Lay& lay, int t)
+    template <class Lay> SP_D static void store(const cpx<R> (&v)[EL], cpx<R>* sm, const Lay& lay, int t)
     {
 #pragma unroll
         for (int m = 0; m < NB; ++m) {
+            if (!has(m, t)) continue;
             const int i = t + T * m;
             const int k = i % P;
             const int base = (i - k) * RAD + k;
@@ -671,6 +688,41 @@ template <class R, int N, bool INV> SP_D int first_element(int t, int j)
     return t + T * (j / R0) + (j % R0) * (N / R0);
 }
 
+template <class R, int N, bool INV, int S, class K, int ST, class Lay>
+SP_D cpx<R>* later_stages(cpx<R> (&v)[PlanOf<K, N>::E], cpx<R>* full, cpx<R>* other, const Lay& lay, const cpx<R>* tws, int t);
+
+// Stage ST, whose inputs are in x, and the stages after it, which leave their outputs in v.
+template <class R, int N, bool INV, int S, bool HALF, class K, int ST, class Lay, int EL>
+SP_D cpx<R>* stage_then(cpx<R> (&x)[EL], cpx<R> (&v)[PlanOf<K, N>::E], cpx<R>* fresh, cpx<R>* other, const Lay& lay,
+                        const cpx<R>* tws, int t)
+{
+    using St = Stage<R, N, INV, ST, K>;
+    St::template compute<S, HALF>(x, tws, t);
+    if constexpr (ST + 1 < PlanOf<K, N>::NS) {
+        St::store(x, fresh, lay, t);
+        __syncthreads();
+        return later_stages<R, N, INV, S, K, ST + 1>(v, fresh, other, lay, tws, t);
+    } else {
+        return fresh;
+    }
+}
+// Stage ST, whose inputs are in `full` behind a barrier, and the stages after it.
+template <class R, int N, bool INV, int S, class K, int ST, class Lay>
+SP_D cpx<R>* later_stages(cpx<R> (&v)[PlanOf<K, N>::E], cpx<R>* full, cpx<R>* other, const Lay& lay, const cpx<R>* tws, int t)
+{
+    using St = Stage<R, N, INV, ST, K>;
+    if constexpr (St::EL == PlanOf<K, N>::E) {
+        St::load(v, full, lay, t);
+        if (other == full) __syncthreads();
+        return stage_then<R, N, INV, S, false, K, ST>(v, v, other, full, lay, tws, t);
+    } else {
+        cpx<R> x[St::EL];
+        St::load(x, full, lay, t);
+        if (other == full) __syncthreads();
+        return stage_then<R, N, INV, S, false, K, ST>(x, v, other, full, lay, tws, t);
+    }
+}
+
 // Run stages [0, NS) of one transform.  On entry v holds the stage-0 inputs (slot
 // j = element first_element(t, j)); on return it holds the last stage's outputs (slot
 // j = element last_element(t, j)).  `fresh` must be safe to write on entry (no reads of
@@ -678,19 +730,8 @@ template <class R, int N, bool INV> SP_D int first_element(int t, int j)
 // each: a buffer is written again only after the barrier that follows every read of it.
 // With other == fresh (one buffer) a second barrier follows each read.  Returns the
 // buffer that is safe to write after the call.  All threads of the block must call this.
-template <class R, int N, bool INV, int S, bool HALF0, class K = R, class Lay, int ST = 0>
-SP_D cpx<R>* run_stages(cpx<R> (&v)[PlanOf<K, N>::E], cpx<R>* fresh, cpx<R>* other, const Lay& lay,
-                        const cpx<R>* tws, int t)
+template <class R, int N, bool INV, int S, bool HALF0, class K = R, class Lay>
+SP_D cpx<R>* run_stages(cpx<R> (&v)[PlanOf<K, N>::E], cpx<R>* fresh, cpx<R>* other, const Lay& lay, const cpx<R>* tws, int t)
 {
-    using St = Stage<R, N, INV, ST, K>;
-    St::template compute<S, HALF0 && ST == 0>(v, tws, t);
-    if constexpr (ST + 1 < PlanOf<K, N>::NS) {
-        St::store(v, fresh, lay, t);
-        __syncthreads();
-        Stage<R, N, INV, ST + 1, K>::load(v, fresh, lay, t);
-        if (other == fresh) __syncthreads();
-        return run_stages<R, N, INV, S, HALF0, K, Lay, ST + 1>(v, other, fresh, lay, tws, t);
-    } else {
-        return fresh;
-    }
+    return stage_then<R, N, INV, S, HALF0, K, 0>(v, v, fresh, other, lay, tws, t);
 }
