@@ -48,10 +48,13 @@ def torch_allocator():
 
 
 def _stream_handle(stream):
+    """The CUDA stream of a torch stream, by default the current one.  Read without making a
+    torch.cuda.Stream (0.3 us instead of 3.1): a 64^3 FP32 solve takes 19 us on the GPU, less
+    than its call took on the host."""
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 class Plan:
@@ -169,9 +172,11 @@ class Plan:
         self._check_io(rho, False)
         if out is None:
             out = torch.empty_like(rho)
-        self._check_io(out, False)
-        self._N.check(self._N.lib.sp_solve(self._h, ctypes.c_void_p(rho.data_ptr()),
-                                           ctypes.c_void_p(out.data_ptr()), _stream_handle(stream)), "sp_solve")
+        else:
+            self._check_io(out, False)
+        rc = self._N.lib.sp_solve(self._h, rho.data_ptr(), out.data_ptr(), _stream_handle(stream))
+        if rc:
+            self._N.check(rc, "sp_solve")
         return out
 
     def _solve_host(self, rho, out, stream):
