@@ -106,37 +106,43 @@ __global__ void k_full_line(int s0, int terms, int nk, double L, const double* a
 }
 
 // ------------------------------------------------------------------------- GEMM
-// C[m][n] = sum_k A[m][k] B[n][k] (both operands K-contiguous), FP64, 32 x 32 tiles, 256
+// C[m][n] = sum_k A[m][k] B[n][k] (both operands K-contiguous), FP64, 32 x 16 tiles, 128
 // threads with 2 x 2 outputs each, K staged through shared memory 16 at a time.  Bound by the
-// FP64 pipe (two FMAs a clock an SM), so small tiles cost nothing in shared-memory reads and
-// waste less at the edges than 64 x 64 ones (129 columns: 160 instead of 192 computed; the
-// last of few waves is shorter).  The epilogue functor receives (m, n, value); skip(m0, n0)
-// names tiles that are not needed.
-constexpr int TM = 32, TN = 32, TK = 16;
+// FP64 pipe (two FMAs a clock an SM, 86 % of it on the tiles that run), so small tiles cost
+// nothing in shared-memory reads and compute less that nobody needs.  Column tiles are aligned
+// to the last column: n + 1 of them are one more than a multiple of 16 at the usual sizes, and
+// the tile that is nearly empty is then the one at column 0, which the symmetric contraction
+// needs least.  Multiplier of a 128^3 grid (129 columns): 2.09 times the entries it needs with
+// 32 x 32 tiles from column 0, 1.19 now.  The epilogue functor receives (m, n, value); skip(m0,
+// n0) names tiles that are not needed.
+constexpr int TM = 32, TN = 16, TK = 16, kGemmThreads = 128;
 
 template <class Epi>
-__global__ void __launch_bounds__(256) k_dgemm_nt(int M, int N, int K, const double* __restrict__ A,
-                                                  long long lda, const double* __restrict__ B,
-                                                  long long ldb, Epi epi)
+__global__ void __launch_bounds__(kGemmThreads) k_dgemm_nt(int M, int N, int K, const double* __restrict__ A,
+                                                           long long lda, const double* __restrict__ B,
+                                                           long long ldb, Epi epi)
 {
     __shared__ double As[TK][TM + 1];
     __shared__ double Bs[TK][TN + 1];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+    const int tx = threadIdx.x % 8, ty = threadIdx.x / 8;
+    const int m0 = blockIdx.y * TM, n0 = N - TN * ((int)blockIdx.x + 1);  // n0 < 0: partly empty
     if (epi.skip(m0, n0)) return;
     double acc[2][2] = {};
     for (int k0 = 0; k0 < K; k0 += TK) {
 #pragma unroll
-        for (int l = threadIdx.x; l < TM * TK; l += 256) {
+        for (int l = threadIdx.x; l < TM * TK; l += kGemmThreads) {
             const int r = l / TK, c = l % TK;
-            const int gm = m0 + r, gn = n0 + r, gk = k0 + c;
-            As[c][r] = (gm < M && gk < K) ? A[(long long)gm * lda + gk] : 0.0;
-            Bs[c][r] = (gn < N && gk < K) ? B[(long long)gn * ldb + gk] : 0.0;
+            As[c][r] = (m0 + r < M && k0 + c < K) ? A[(long long)(m0 + r) * lda + k0 + c] : 0.0;
+        }
+#pragma unroll
+        for (int l = threadIdx.x; l < TN * TK; l += kGemmThreads) {
+            const int r = l / TK, c = l % TK;
+            Bs[c][r] = (n0 + r >= 0 && k0 + c < K) ? B[(long long)(n0 + r) * ldb + k0 + c] : 0.0;
         }
         __syncthreads();
 #pragma unroll
         for (int c = 0; c < TK; ++c) {
-            const double a0 = As[c][ty], a1 = As[c][ty + 16], b0 = Bs[c][tx], b1 = Bs[c][tx + 16];
+            const double a0 = As[c][ty], a1 = As[c][ty + 16], b0 = Bs[c][tx], b1 = Bs[c][tx + 8];
             acc[0][0] = fma(a0, b0, acc[0][0]);
             acc[0][1] = fma(a0, b1, acc[0][1]);
             acc[1][0] = fma(a1, b0, acc[1][0]);
@@ -148,8 +154,8 @@ __global__ void __launch_bounds__(256) k_dgemm_nt(int M, int N, int K, const dou
     for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const int gm = m0 + ty + 16 * i, gn = n0 + tx + 16 * j;
-            if (gm < M && gn < N) epi(gm, gn, acc[i][j]);
+            const int gm = m0 + ty + 16 * i, gn = n0 + tx + 8 * j;
+            if (gm < M && gn >= 0) epi(gm, gn, acc[i][j]);
         }
 }
 
@@ -179,19 +185,19 @@ __device__ __forceinline__ double parts_value(int which, int k, double kap, doub
 }
 
 // The quadrature sums of one axis, all four (direct and by-parts integrands of G and H) in
-// one launch: 16 x 16 outputs (s, k) a block, blockIdx.z = 0 for G, 1 for H.  A block runs
+// one launch: 16 x 8 outputs (s, k) a block, blockIdx.z = 0 for G, 1 for H.  A block runs
 // the direct sum, the by-parts sum, or (where the border between them crosses it) both.
 // Bound by the FP64 pipe at two FMAs a clock an SM, so the tile is small: it fills the chip
-// (486 blocks at n = 128, where 64 x 64 tiles gave 21), and two shared-memory reads an FMA
-// do not show.  At n = 128 the four sums took 9.5 ms as four GEMMs.
-constexpr int kAxT = 16, kAxK = 32;
-__global__ void __launch_bounds__(kAxT * kAxT) k_axis_sums(int rows, int nk, int nq, const double* __restrict__ E,
+// (918 blocks at n = 128, where 64 x 64 tiles gave 21) and few blocks run both sums, and
+// two shared-memory reads an FMA do not show.
+constexpr int kAxS = 16, kAxC = 8, kAxK = 32;
+__global__ void __launch_bounds__(kAxS * kAxC) k_axis_sums(int rows, int nk, int nq, const double* __restrict__ E,
                                                            const double* __restrict__ C, const double* __restrict__ a, double L,
                                                            double* __restrict__ G, double* __restrict__ H)
 {
-    __shared__ double As[kAxT][kAxK + 1], Bs[kAxT][kAxK + 1];
-    const int which = blockIdx.z, tx = threadIdx.x % kAxT, ty = threadIdx.x / kAxT;
-    const int s = blockIdx.y * kAxT + ty, k = blockIdx.x * kAxT + tx;
+    __shared__ double As[kAxS][kAxK + 1], Bs[kAxC][kAxK + 1];
+    const int which = blockIdx.z, tx = threadIdx.x % kAxC, ty = threadIdx.x / kAxC;
+    const int s = blockIdx.y * kAxS + ty, k = blockIdx.x * kAxC + tx;
     const bool in = s < rows && k < nk;
     const double al = in ? a[s] : 1.0, kap = kPi * k / L;
     const bool parts = in && by_parts(k, kap, al);
@@ -201,11 +207,11 @@ __global__ void __launch_bounds__(kAxT * kAxT) k_axis_sums(int rows, int nk, int
         const double* A = E + (2 * form + which) * rn;
         double acc = 0.0;
         for (int q0 = 0; q0 < nq; q0 += kAxK) {
-            for (int l = threadIdx.x; l < kAxT * kAxK; l += kAxT * kAxT) {
+            for (int l = threadIdx.x; l < (kAxS + kAxC) * kAxK; l += kAxS * kAxC) {
                 const int r = l / kAxK, c = l % kAxK, q = q0 + c;
-                const int gs = blockIdx.y * kAxT + r, gk = blockIdx.x * kAxT + r;
-                As[r][c] = gs < rows && q < nq ? A[(long long)gs * nq + q] : 0.0;
-                Bs[r][c] = gk < nk && q < nq ? C[(long long)gk * nq + q] : 0.0;
+                const int gs = blockIdx.y * kAxS + r, gk = blockIdx.x * kAxC + r - kAxS;
+                if (r < kAxS) As[r][c] = gs < rows && q < nq ? A[(long long)gs * nq + q] : 0.0;
+                else Bs[r - kAxS][c] = gk < nk && q < nq ? C[(long long)gk * nq + q] : 0.0;
             }
             __syncthreads();
             double part = 0.0;  // summed by steps: the rounding of nq terms in a row stays below the rule's
@@ -370,46 +376,47 @@ __global__ void k_period_rows(int n, int F, double* T)
     T[idx] = (k == 0 || k == n ? 0.5 : 1.0) * d / (double)F;
 }
 
-// C[b][m][j] = sum_k A[m][k] B[b][k][j]: the change of period along a strided axis (FP64,
-// tiles as in k_dgemm_nt).  B's rows have stride ldb, its batches sb; C's likewise.
-__global__ void __launch_bounds__(256) k_dgemm_nn(int M, int N, int K, const double* __restrict__ A,
-                                                  const double* __restrict__ B, long long ldb, long long sb,
-                                                  double* __restrict__ C, long long ldc, long long sc)
+// C[b][m][j] = sum_k A[m][k] B[b][k][j]: the change of period along a strided axis (FP64).
+// B's rows have stride ldb, its batches sb; C's likewise.  Bound by the FP64 pipe; 16 x 16 tiles
+// (64 threads, 2 x 2 outputs each) keep the waste at the edges small (F/2 + 1 rows are one more
+// than a multiple of 16 at most lengths) and give an 83^3 grid 2400 blocks a launch, where
+// 64 x 64 tiles gave 168 to 194, one to two an SM.
+constexpr int kNnT = 16;
+__global__ void __launch_bounds__(64) k_dgemm_nn(int M, int N, int K, const double* __restrict__ A,
+                                                 const double* __restrict__ B, long long ldb, long long sb,
+                                                 double* __restrict__ C, long long ldc, long long sc)
 {
-    __shared__ double As[16][65];
-    __shared__ double Bs[16][64];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+    __shared__ double As[kNnT][kNnT + 1];
+    __shared__ double Bs[kNnT][kNnT];
+    const int tx = threadIdx.x % 8, ty = threadIdx.x / 8;
+    const int m0 = blockIdx.y * kNnT, n0 = blockIdx.x * kNnT;
     B += blockIdx.z * sb;
     C += blockIdx.z * sc;
-    double acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int l = threadIdx.x; l < 1024; l += 256) {
-            const int r = l / 16, c = l % 16;
+    double acc[2][2] = {};
+    for (int k0 = 0; k0 < K; k0 += kNnT) {
+#pragma unroll
+        for (int l = threadIdx.x; l < kNnT * kNnT; l += 64) {
+            const int r = l / kNnT, c = l % kNnT;
             As[c][r] = (m0 + r < M && k0 + c < K) ? A[(long long)(m0 + r) * K + k0 + c] : 0.0;
-            const int kr = l / 64, nc = l % 64;
-            Bs[kr][nc] = (k0 + kr < K && n0 + nc < N) ? B[(long long)(k0 + kr) * ldb + n0 + nc] : 0.0;
+            Bs[r][c] = (k0 + r < K && n0 + c < N) ? B[(long long)(k0 + r) * ldb + n0 + c] : 0.0;
         }
         __syncthreads();
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-            double av[4], bv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) av[i] = As[c][ty + 16 * i];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) bv[i] = Bs[c][tx + 16 * i];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+        for (int c = 0; c < kNnT; ++c) {
+            const double a0 = As[c][ty], a1 = As[c][ty + 8], b0 = Bs[c][tx], b1 = Bs[c][tx + 8];
+            acc[0][0] = fma(a0, b0, acc[0][0]);
+            acc[0][1] = fma(a0, b1, acc[0][1]);
+            acc[1][0] = fma(a1, b0, acc[1][0]);
+            acc[1][1] = fma(a1, b1, acc[1][1]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (m0 + ty + 16 * i < M && n0 + tx + 16 * j < N) C[(long long)(m0 + ty + 16 * i) * ldc + n0 + tx + 16 * j] = acc[i][j];
+        for (int j = 0; j < 2; ++j)
+            if (m0 + ty + 8 * i < M && n0 + tx + 8 * j < N)
+                C[(long long)(m0 + ty + 8 * i) * ldc + n0 + tx + 8 * j] = acc[i][j];
 }
 
 struct EpiStore {
@@ -462,9 +469,11 @@ static sp_status setup_axis(sp_plan p, int ax, cudaStream_t st)
             s_split, S, nk, L, p->d_gs_a, p->d_G[ax], p->d_H[ax]);
     }
     if (s_split > 0) {
-        // panels: a panel spans a phase of at most 2 pi of cos(pi k y / L), k <= n, where the
-        // 16-point rule's error is below 1e-28 of the panel's integrand
-        const int P = n > 32 ? (n + 1) / 2 : (n > 8 ? n : 8), Q = kGLQ;
+        // panels: a panel spans a phase of at most 3 pi of cos(pi k y / L), k <= n.  The 16-point
+        // rule's error is phi^33 (16!)^4 / (33 (32!)^3) of the integrand's 32nd derivative, phi
+        // the phase: 5e-23 for the cosine alone, below 1e-17 with the Gaussian's own variation
+        // over a panel (a L^2 < 40: at most 4.2 more of phase at n = 33)
+        const int P = n > 32 ? (n + 2) / 3 : (n > 8 ? n : 8), Q = kGLQ;
         const long long nq = (long long)P * Q;
         DevBuf nodes(st), E(st), C(st);
         const long long rn = (long long)s_split * nq;
@@ -476,8 +485,8 @@ static sp_status setup_axis(sp_plan p, int ax, cudaStream_t st)
         k_nodes<<<nblk(nq, 256), 256, 0, st>>>(P, L, tpos, y, wq);
         k_gauss_rows<<<nblk(rn, 256), 256, 0, st>>>(s_split, (int)nq, p->d_gs_a, y, wq, E0, E2, F0, F2);
         k_cos_rows<<<nblk(nk * nq, 256), 256, 0, st>>>(nk, P, Q, tpos, C.d());
-        dim3 grid(nblk(nk, kAxT), nblk(s_split, kAxT), 2);
-        k_axis_sums<<<grid, kAxT * kAxT, 0, st>>>(s_split, nk, (int)nq, E0, C.d(), p->d_gs_a, L, p->d_G[ax], p->d_H[ax]);
+        dim3 grid(nblk(nk, kAxC), nblk(s_split, kAxS), 2);
+        k_axis_sums<<<grid, kAxS * kAxC, 0, st>>>(s_split, nk, (int)nq, E0, C.d(), p->d_gs_a, L, p->d_G[ax], p->d_H[ax]);
         rc = sp_cuda_check(cudaGetLastError(), "setup: 1D integral kernels");
         if (rc) return rc;
     }
@@ -534,15 +543,15 @@ static sp_status setup_period(sp_plan p, cudaStream_t st)
         double* next = X.d();
         if (T2.p) {
             dim3 grid(nblk(cols, TN), nblk((long long)n0p * n1p, TM));
-            k_dgemm_nt<<<grid, 256, 0, st>>>(n0p * n1p, cols, n2p, p->d_M64, (long long)p->ldz,
+            k_dgemm_nt<<<grid, kGemmThreads, 0, st>>>(n0p * n1p, cols, n2p, p->d_M64, (long long)p->ldz,
                                              T2.d() + (long long)c0 * n2p, (long long)n2p, EpiStore{next, CW});
             cur = next;
             ld = CW;
             next = Y.d();
         }
         if (T0.p) {
-            dim3 grid(1, nblk(q0, 64), n1p);
-            k_dgemm_nn<<<grid, 256, 0, st>>>(q0, cols, n0p, T0.d(), cur, ld, ld * n0p, next, CW, (long long)CW * q0);
+            dim3 grid(nblk(cols, kNnT), nblk(q0, kNnT), n1p);
+            k_dgemm_nn<<<grid, 64, 0, st>>>(q0, cols, n0p, T0.d(), cur, ld, ld * n0p, next, CW, (long long)CW * q0);
             cur = next;
             ld = CW;
             next = cur == X.d() ? Y.d() : X.d();
@@ -550,11 +559,11 @@ static sp_status setup_period(sp_plan p, cudaStream_t st)
         if (T1.p) {  // rows (k0', column) of one k1 are contiguous, or ld apart without an earlier step
             const long long w = (long long)q0 * ld;
             if (ld == CW) {
-                dim3 grid(nblk(w, 64), nblk(q1, 64));
-                k_dgemm_nn<<<grid, 256, 0, st>>>(q1, (int)w, n1p, T1.d(), cur, w, 0, next, w, 0);
+                dim3 grid(nblk(w, kNnT), nblk(q1, kNnT));
+                k_dgemm_nn<<<grid, 64, 0, st>>>(q1, (int)w, n1p, T1.d(), cur, w, 0, next, w, 0);
             } else {
-                dim3 grid(1, nblk(q1, 64), q0);  // one k0 at a time: batch stride ld
-                k_dgemm_nn<<<grid, 256, 0, st>>>(q1, cols, n1p, T1.d(), cur, w, ld, next, (long long)CW * q0, CW);
+                dim3 grid(nblk(cols, kNnT), nblk(q1, kNnT), q0);  // one k0 at a time: batch stride ld
+                k_dgemm_nn<<<grid, 64, 0, st>>>(q1, cols, n1p, T1.d(), cur, w, ld, next, (long long)CW * q0, CW);
                 ld = CW;
             }
             cur = next;
@@ -642,7 +651,7 @@ sp_status sp_setup_run(sp_plan p, cudaStream_t st)
                 k_mult_lhs<<<dim3(nblk(2 * S, 256), rows), 256, 0, st>>>((int)r0, S, n0p, sym, p->d_gs_w, bt[0], bt[1], Ap.d());
             epi.row0 = (int)r0;
             dim3 grid(nblk(n2p, TN), nblk(rows, TM));
-            k_dgemm_nt<<<grid, 256, 0, st>>>(rows, n2p, K, Ap.d(), K, bt[2], 2 * S, epi);
+            k_dgemm_nt<<<grid, kGemmThreads, 0, st>>>(rows, n2p, K, Ap.d(), K, bt[2], 2 * S, epi);
         }
         if (cube) k_cube_fill<<<nblk((long long)n0p * n0p * n0p, 256), 256, 0, st>>>(n0p, p->ldz, p->d_M64);
         const long long mcount = (long long)n0p * n1p * p->ldz;
