@@ -106,16 +106,19 @@ __global__ void k_full_line(int s0, int terms, int nk, double L, const double* a
 }
 
 // ------------------------------------------------------------------------- GEMM
-// C[m][n] = sum_k A[m][k] B[n][k] (both operands K-contiguous), FP64, 32 x 16 tiles, 128
+// C[m][n] = sum_k A[m][k] B[n][k] (both operands K-contiguous), FP64, 16 x 16 tiles, 64
 // threads with 2 x 2 outputs each, K staged through shared memory 16 at a time.  Bound by the
-// FP64 pipe (two FMAs a clock an SM, 86 % of it on the tiles that run), so small tiles cost
-// nothing in shared-memory reads and compute less that nobody needs.  Column tiles are aligned
+// FP64 pipe (two FMAs a clock an SM), so small tiles cost nothing in shared-memory reads,
+// compute less that nobody needs and spread evenly over the SMs.  Column tiles are aligned
 // to the last column: n + 1 of them are one more than a multiple of 16 at the usual sizes, and
 // the tile that is nearly empty is then the one at column 0, which the symmetric contraction
-// needs least.  Multiplier of a 128^3 grid (129 columns): 2.09 times the entries it needs with
-// 32 x 32 tiles from column 0, 1.19 now.  The epilogue functor receives (m, n, value); skip(m0,
-// n0) names tiles that are not needed.
-constexpr int TM = 32, TN = 16, TK = 16, kGemmThreads = 128;
+// needs least.  Multiplier of a 128^3 grid (129 columns): 32 x 32 tiles from column 0 computed
+// 2.09 times the entries it needs (1616 us), 32 x 16 from the last 1.19 times (1083 us, 5.6
+// tiles an SM), these 1.18 times (955 us).  Row tiles are blockIdx.x (there are up to 65664):
+// blocks of one column tile run together, and the skipped ones of the low columns last (columns
+// fastest: precompute 1.58 ms instead of 1.40).  The epilogue functor receives (m, n, value);
+// skip(m0, n0) names tiles that are not needed.
+constexpr int TM = 16, TN = 16, TK = 16, kGemmThreads = 64;
 
 template <class Epi>
 __global__ void __launch_bounds__(kGemmThreads) k_dgemm_nt(int M, int N, int K, const double* __restrict__ A,
@@ -125,7 +128,7 @@ __global__ void __launch_bounds__(kGemmThreads) k_dgemm_nt(int M, int N, int K, 
     __shared__ double As[TK][TM + 1];
     __shared__ double Bs[TK][TN + 1];
     const int tx = threadIdx.x % 8, ty = threadIdx.x / 8;
-    const int m0 = blockIdx.y * TM, n0 = N - TN * ((int)blockIdx.x + 1);  // n0 < 0: partly empty
+    const int m0 = blockIdx.x * TM, n0 = N - TN * ((int)blockIdx.y + 1);  // n0 < 0: partly empty
     if (epi.skip(m0, n0)) return;
     double acc[2][2] = {};
     for (int k0 = 0; k0 < K; k0 += TK) {
@@ -142,7 +145,7 @@ __global__ void __launch_bounds__(kGemmThreads) k_dgemm_nt(int M, int N, int K, 
         __syncthreads();
 #pragma unroll
         for (int c = 0; c < TK; ++c) {
-            const double a0 = As[c][ty], a1 = As[c][ty + 16], b0 = Bs[c][tx], b1 = Bs[c][tx + 8];
+            const double a0 = As[c][ty], a1 = As[c][ty + 8], b0 = Bs[c][tx], b1 = Bs[c][tx + 8];
             acc[0][0] = fma(a0, b0, acc[0][0]);
             acc[0][1] = fma(a0, b1, acc[0][1]);
             acc[1][0] = fma(a1, b0, acc[1][0]);
@@ -154,7 +157,7 @@ __global__ void __launch_bounds__(kGemmThreads) k_dgemm_nt(int M, int N, int K, 
     for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const int gm = m0 + ty + 16 * i, gn = n0 + tx + 8 * j;
+            const int gm = m0 + ty + 8 * i, gn = n0 + tx + 8 * j;
             if (gm < M && gn >= 0) epi(gm, gn, acc[i][j]);
         }
 }
@@ -542,7 +545,7 @@ static sp_status setup_period(sp_plan p, cudaStream_t st)
         long long ld = p->ldz;
         double* next = X.d();
         if (T2.p) {
-            dim3 grid(nblk(cols, TN), nblk((long long)n0p * n1p, TM));
+            dim3 grid(nblk((long long)n0p * n1p, TM), nblk(cols, TN));
             k_dgemm_nt<<<grid, kGemmThreads, 0, st>>>(n0p * n1p, cols, n2p, p->d_M64, (long long)p->ldz,
                                              T2.d() + (long long)c0 * n2p, (long long)n2p, EpiStore{next, CW});
             cur = next;
@@ -650,7 +653,7 @@ sp_status sp_setup_run(sp_plan p, cudaStream_t st)
             else
                 k_mult_lhs<<<dim3(nblk(2 * S, 256), rows), 256, 0, st>>>((int)r0, S, n0p, sym, p->d_gs_w, bt[0], bt[1], Ap.d());
             epi.row0 = (int)r0;
-            dim3 grid(nblk(n2p, TN), nblk(rows, TM));
+            dim3 grid(nblk(rows, TM), nblk(n2p, TN));
             k_dgemm_nt<<<grid, kGemmThreads, 0, st>>>(rows, n2p, K, Ap.d(), K, bt[2], 2 * S, epi);
         }
         if (cube) k_cube_fill<<<nblk((long long)n0p * n0p * n0p, 256), 256, 0, st>>>(n0p, p->ldz, p->d_M64);
