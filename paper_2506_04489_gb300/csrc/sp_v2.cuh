@@ -95,9 +95,13 @@ template <class R, int PER> struct LayStrided {
 };
 // first radix of plan K's transforms (the inverse's is the forward's last)
 template <class K, int N, bool INV> constexpr int first_radix() { return radix_at<K, N, INV>(0); }
+// A first radix of 2 at 1024 and above keeps 8: a padding row after every second one makes the
+// buffers half as large again and takes a resident CTA (512^3 double-float x pass, ms, after
+// every 2 rows against 8: 12.8 / 10.9; FP32 at 1536 258 / 235 us in x, 74 / 94 in y inverse).
 template <class K, int N, bool INV> constexpr int strided_per()
 {
-    return first_radix<K, N, INV>() % 2 == 0 ? first_radix<K, N, INV>() : 0;
+    constexpr int r = first_radix<K, N, INV>();
+    return r % 2 ? 0 : (r == 2 && N >= 1024 ? 8 : r);
 }
 template <class R, class K, int N, bool INV> using LayLines = LayStrided<R, strided_per<K, N, INV>()>;
 // entries of an exchange buffer of B strided lines, whichever direction uses it
@@ -185,7 +189,7 @@ template <class R, int N> constexpr int lanes_b_max()
 // barriers and balance better, down to where half-used sectors and idle lanes cost more.
 // Double-float 4 columns, FP64 2 from 128 up (x passes, us, 8 columns against this: double-
 // float 128^3 129 / 117, 256^3 1065 / 1003, FP64 32^3 20.8 / 16.5, 128^3 788 / 745, 256^3
-// 7034 / 6536); at 1024 (4 at most) the x pass takes 2 (512^3 14.2 / 12.8 ms) and the
+// 7034 / 6536); at 1024 (4 at most) the x pass takes 2 (512^3 11.5 / 10.9 ms) and the
 // double-float y passes at 512 stay at 8 (293/282 against 306/299).  FP32: 8 columns, the
 // pipelined kernel's tile; at 1024 the x and y forward passes are faster without the pipeline
 // on 8 (16 warps an SM, 64-byte rows) than with it on 4 (8 warps): 512^3 x 3.66 / 1.96 ms, y
