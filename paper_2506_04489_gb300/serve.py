@@ -51,7 +51,7 @@ def transform_length(n: int, precision: str) -> int:
     N = 2 * n
     if N in TUNED_LENGTHS:
         return N
-    F = next(f for f in F_LENGTHS if f >= N)
+    F = next((f for f in F_LENGTHS if f >= N), N)  # no plan takes 2n > 2048
     m = N
     for p in (2, 3, 5, 7):
         while m % p == 0:
