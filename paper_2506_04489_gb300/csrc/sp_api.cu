@@ -158,6 +158,111 @@ extern "C" sp_status sp_plan_create_ex(sp_plan* out, const int n[3], const doubl
     return create_plan(out, n, box_lo, box_hi, padding, gs_w, gs_a, gs_terms, eps, prec, max_batch, allocator, false);
 }
 
+// What the sizes of a plan's buffers depend on: lengths, strides and the GS table's length
+// (0 gs_terms: generated).  Host only.
+static void plan_geometry(sp_plan p, const int n[3], const double box_lo[3], const double box_hi[3], int gs_terms,
+                          double eps, sp_precision prec, int max_batch, bool may_embed)
+{
+    for (int ax = 0; ax < 3; ++ax) {
+        p->n[ax] = n[ax];
+        p->N[ax] = 2 * n[ax];
+        p->lo[ax] = box_lo[ax];
+        p->hi[ax] = box_hi[ax];
+        p->h[ax] = (box_hi[ax] - box_lo[ax]) / (n[ax] - 1);
+        p->L[ax] = n[ax] * p->h[ax];
+        // a padded length with a prime factor above 7 has no radix plan: Bluestein's
+        // algorithm, a circular convolution of length M = 2^k >= 2N - 1
+        if (!sp_radix_plan(p->N[ax], &p->rp[ax])) {
+            p->rp[ax].nst = 0;
+            int M = 1;
+            while (M < 2 * p->N[ax] - 1) M *= 2;
+            p->blue_M[ax] = M;
+            sp_radix_plan(M, &p->blue_rp[ax]);
+        }
+    }
+    p->prec = prec;
+    p->max_batch = max_batch;
+    p->ldz = (n[2] + 1 + 7) & ~7;
+    p->plane = 2LL * n[1] * p->ldz;
+    const size_t csize = (prec == SP_FP64 || prec == SP_DF32) ? 16 : 8;
+    p->emb = sp_embeds(p->N, prec, p->F) && may_embed;
+    if (!p->emb)
+        for (int ax = 0; ax < 3; ++ax) p->F[ax] = p->N[ax];
+    p->ldf = (p->F[2] / 2 + 1 + 7) & ~7;
+    p->planef = (long long)p->F[1] * p->ldf;
+    p->keep_n = p->emb && csize * n[0] * p->plane <= SP_NOALLOC_MAX_BYTES && csize * n[0] * p->planef > SP_NOALLOC_MAX_BYTES;
+    p->work_bytes = csize * (size_t)max_batch * n[0] * (size_t)p->planef;
+    p->eps = eps;
+    p->delta = sqrt(p->L[0] * p->L[0] + p->L[1] * p->L[1] + p->L[2] * p->L[2]);
+    p->h_tau = 0.1;
+    p->eta = 1e-17;
+    p->gs_user = gs_terms > 0;
+    // the generated table's length is fixed by eps and delta (eq. sin_1_x): known now
+    p->gs_cap = p->gs_terms = p->gs_user ? gs_terms : sp_gs_terms(p);
+}
+
+// Every device buffer that a plan holds, in the order of allocation: visit(pointer, bytes,
+// name) for each, up to the first failure.  The one list behind creation and sp_plan_bytes.
+template <class Visit> static sp_status plan_buffers(sp_plan p, Visit&& visit)
+{
+    sp_status rc;
+#define SP_BUFFER(ptr, bytes) \
+    if ((rc = visit((void**)&(ptr), (size_t)(bytes), #ptr))) return rc
+    const size_t csize = (p->prec == SP_FP64 || p->prec == SP_DF32) ? 16 : 8;
+    SP_BUFFER(p->d_status, 256);
+    SP_BUFFER(p->d_gs_w, sizeof(double) * p->gs_cap);
+    SP_BUFFER(p->d_gs_a, sizeof(double) * p->gs_cap);
+    // 1D integral tables [s][k] per axis; axes with the same (n, L) share one
+    for (int ax = 0; ax < 3; ++ax) {
+        int same = -1;
+        for (int q = 0; q < ax; ++q)
+            if (p->n[q] == p->n[ax] && p->L[q] == p->L[ax]) { same = q; break; }
+        if (same >= 0) {
+            p->d_G[ax] = p->d_G[same];
+            p->d_H[ax] = p->d_H[same];
+            continue;
+        }
+        const size_t tb = sizeof(double) * (size_t)p->gs_cap * (p->n[ax] + 1);
+        SP_BUFFER(p->d_G[ax], tb);
+        SP_BUFFER(p->d_H[ax], tb);
+    }
+    const size_t mcount = (size_t)(p->n[0] + 1) * (p->n[1] + 1) * p->ldz;
+    SP_BUFFER(p->d_M64, sizeof(double) * mcount);
+    if (!p->emb || p->keep_n) {
+        if (p->prec == SP_FP32 || p->prec == SP_MIXED) SP_BUFFER(p->d_M32, sizeof(float) * mcount);
+        if (p->prec == SP_DF32) SP_BUFFER(p->d_Mdf, sizeof(df32) * mcount);
+    }
+    if (p->emb) {
+        SP_BUFFER(p->d_Ms, csize / 2 * (size_t)(p->F[0] / 2 + 1) * (p->F[1] / 2 + 1) * p->ldf);
+        for (int ax = 0; ax < 3; ++ax)
+            if (!sp_v2_supported(p->N[ax])) SP_BUFFER(p->d_twF[ax], csize * (p->F[ax] + SP_TW_STAGED_MAX));
+    }
+    for (int ax = 0; ax < 3; ++ax) {
+        SP_BUFFER(p->d_tw64[ax], sizeof(cpx<double>) * p->N[ax]);
+        SP_BUFFER(p->d_tw32[ax], sizeof(cpx<float>) * (p->N[ax] + SP_TW_STAGED_MAX));
+        SP_BUFFER(p->d_twdf[ax], sizeof(cpx<df32>) * (p->N[ax] + SP_TW_STAGED_MAX));
+    }
+    for (int ax = 0; ax < 3; ++ax)
+        if (p->blue_M[ax]) SP_BUFFER(p->d_blue[ax], sp_bluestein_bytes(p, ax));
+    SP_BUFFER(p->d_work, p->work_bytes);
+#undef SP_BUFFER
+    return SP_OK;
+}
+
+size_t sp_plan_bytes(const int n[3], const double box_lo[3], const double box_hi[3], double eps, sp_precision prec,
+                     int max_batch, bool may_embed)
+{
+    sp_plan_s view = {};
+    plan_geometry(&view, n, box_lo, box_hi, 0, eps, prec, max_batch, may_embed);
+    if (view.gs_cap < 1 || view.gs_cap > kGsCap) view.gs_cap = 0;  // creation refuses the plan
+    size_t total = 0;
+    plan_buffers(&view, [&](void**, size_t bytes, const char*) {
+        total += bytes;
+        return SP_OK;
+    });
+    return total;
+}
+
 static sp_status create_plan(sp_plan* out, const int n[3], const double box_lo[3],
                              const double box_hi[3], int padding, const double* gs_w,
                              const double* gs_a, int gs_terms, double eps,
@@ -197,47 +302,12 @@ static sp_status create_plan(sp_plan* out, const int n[3], const double box_lo[3
         p->alloc = *allocator;
         p->has_alloc = true;
     }
-    for (int ax = 0; ax < 3; ++ax) {
-        p->n[ax] = n[ax];
-        p->N[ax] = 2 * n[ax];
-        p->lo[ax] = box_lo[ax];
-        p->hi[ax] = box_hi[ax];
-        p->h[ax] = (box_hi[ax] - box_lo[ax]) / (n[ax] - 1);
-        p->L[ax] = n[ax] * p->h[ax];
-        // a padded length with a prime factor above 7 has no radix plan: Bluestein's
-        // algorithm, a circular convolution of length M = 2^k >= 2N - 1
-        if (!sp_radix_plan(p->N[ax], &p->rp[ax])) {
-            p->rp[ax].nst = 0;
-            int M = 1;
-            while (M < 2 * p->N[ax] - 1) M *= 2;
-            p->blue_M[ax] = M;
-            sp_radix_plan(M, &p->blue_rp[ax]);
-        }
-    }
-    p->prec = prec;
-    p->max_batch = max_batch;
-    p->ldz = (n[2] + 1 + 7) & ~7;
-    p->plane = 2LL * n[1] * p->ldz;
-    const size_t csize = (prec == SP_FP64 || prec == SP_DF32) ? 16 : 8;
-    p->emb = sp_embeds(p->N, prec, p->F) && may_embed;
-    if (!p->emb)
-        for (int ax = 0; ax < 3; ++ax) p->F[ax] = p->N[ax];
-    p->ldf = (p->F[2] / 2 + 1 + 7) & ~7;
-    p->planef = (long long)p->F[1] * p->ldf;
-    p->keep_n = p->emb && csize * n[0] * p->plane <= SP_NOALLOC_MAX_BYTES && csize * n[0] * p->planef > SP_NOALLOC_MAX_BYTES;
-    p->eps = eps;
-    p->delta = sqrt(p->L[0] * p->L[0] + p->L[1] * p->L[1] + p->L[2] * p->L[2]);
-    p->h_tau = 0.1;
-    p->eta = 1e-17;
-    p->gs_user = user;
-    // the generated table's length is fixed by eps and delta (eq. sin_1_x): known now
-    const int terms = user ? gs_terms : sp_gs_terms(p);
+    plan_geometry(p, n, box_lo, box_hi, user ? gs_terms : 0, eps, prec, max_batch, may_embed);
+    const int terms = p->gs_terms;
     if (!user && (terms < 1 || terms > kGsCap)) {
         delete p;
         return sp_fail(SP_ERR_INVALID, "GS table of %d terms (eps %g): at most %d", terms, eps, kGsCap);
     }
-    p->gs_cap = terms;
-    p->gs_terms = terms;
 
     p->ev = new (std::nothrow) std::vector<cudaEvent_t>();
     p->h_gs_a = (double*)malloc(sizeof(double) * p->gs_cap);
@@ -259,49 +329,12 @@ static sp_status create_plan(sp_plan* out, const int n[3], const double box_lo[3
         free_plan(p);
         return rc;
     }
-#define SP_ALLOC(ptr, bytes)                                                           \
-    do {                                                                               \
-        if ((rc = sp_plan_alloc(p, (void**)&(ptr), (bytes), #ptr))) {                  \
-            free_plan(p);                                                              \
-            return rc;                                                                 \
-        }                                                                              \
-    } while (0)
-    SP_ALLOC(p->d_status, 256);
-    SP_ALLOC(p->d_gs_w, sizeof(double) * p->gs_cap);
-    SP_ALLOC(p->d_gs_a, sizeof(double) * p->gs_cap);
-    // 1D integral tables [s][k] per axis; axes with the same (n, L) share one
-    for (int ax = 0; ax < 3; ++ax) {
-        int same = -1;
-        for (int q = 0; q < ax; ++q)
-            if (p->n[q] == p->n[ax] && p->L[q] == p->L[ax]) { same = q; break; }
-        if (same >= 0) {
-            p->d_G[ax] = p->d_G[same];
-            p->d_H[ax] = p->d_H[same];
-            continue;
-        }
-        const size_t tb = sizeof(double) * (size_t)p->gs_cap * (n[ax] + 1);
-        SP_ALLOC(p->d_G[ax], tb);
-        SP_ALLOC(p->d_H[ax], tb);
-    }
-    const size_t mcount = (size_t)(n[0] + 1) * (n[1] + 1) * p->ldz;
-    SP_ALLOC(p->d_M64, sizeof(double) * mcount);
-    if (!p->emb || p->keep_n) {
-        if (prec == SP_FP32 || prec == SP_MIXED) SP_ALLOC(p->d_M32, sizeof(float) * mcount);
-        if (prec == SP_DF32) SP_ALLOC(p->d_Mdf, sizeof(df32) * mcount);
-    }
-    if (p->emb) {
-        SP_ALLOC(p->d_Ms, csize / 2 * (size_t)(p->F[0] / 2 + 1) * (p->F[1] / 2 + 1) * p->ldf);
-        for (int ax = 0; ax < 3; ++ax)
-            if (!sp_v2_supported(p->N[ax])) SP_ALLOC(p->d_twF[ax], csize * (p->F[ax] + SP_TW_STAGED_MAX));
-    }
-    for (int ax = 0; ax < 3; ++ax) {
-        SP_ALLOC(p->d_tw64[ax], sizeof(cpx<double>) * p->N[ax]);
-        SP_ALLOC(p->d_tw32[ax], sizeof(cpx<float>) * (p->N[ax] + SP_TW_STAGED_MAX));
-        SP_ALLOC(p->d_twdf[ax], sizeof(cpx<df32>) * (p->N[ax] + SP_TW_STAGED_MAX));
+    if ((rc = plan_buffers(p, [p](void** ptr, size_t bytes, const char* what) { return sp_plan_alloc(p, ptr, bytes, what); }))) {
+        free_plan(p);
+        return rc;
     }
     for (int ax = 0; ax < 3; ++ax) {  // Bluestein tables: built on the host, copied once
         if (!p->blue_M[ax]) continue;
-        SP_ALLOC(p->d_blue[ax], sp_bluestein_bytes(p, ax));
         std::vector<unsigned char> host(sp_bluestein_bytes(p, ax));
         sp_bluestein_fill(p, ax, host.data());
         // pageable source: the call returns once the bytes are staged, so host may go
@@ -313,9 +346,6 @@ static sp_status create_plan(sp_plan* out, const int n[3], const double box_lo[3
             return rc;
         }
     }
-    p->work_bytes = csize * (size_t)max_batch * n[0] * (size_t)p->planef;
-    SP_ALLOC(p->d_work, p->work_bytes);
-#undef SP_ALLOC
     const cudaError_t ce = p->mem_st ? cudaMemsetAsync(p->d_status, 0, 256, p->mem_st) : cudaMemset(p->d_status, 0, 256);
     if ((rc = sp_cuda_check(ce == cudaSuccess && p->mem_st ? cudaStreamSynchronize(p->mem_st) : ce,
                             "clear status word"))) {

@@ -125,11 +125,15 @@ struct sp_plan_s {
 sp_status sp_mark(sp_plan p, cudaStream_t st);
 // Record the plan's completion event on `st` after work issued there.
 sp_status sp_record_done(sp_plan p, cudaStream_t st);
-// Device allocation owned by the plan (the caller's allocator, else cudaMalloc).
 // Host-built Bluestein table of one axis (layout above), in the plan's arithmetic type:
 // bytes, and the fill into a host buffer of that size.
 size_t sp_bluestein_bytes(const sp_plan_s* p, int ax);
 void sp_bluestein_fill(const sp_plan_s* p, int ax, void* host);
+// Device bytes that a plan with a generated GS table holds (host only): the sum of its
+// buffers, on the lengths F where sp_embeds says so and may_embed, else on 2n.
+size_t sp_plan_bytes(const int n[3], const double box_lo[3], const double box_hi[3], double eps, sp_precision prec,
+                     int max_batch, bool may_embed);
+// Device allocation owned by the plan (the caller's allocator, else cudaMallocAsync).
 sp_status sp_plan_alloc(sp_plan p, void** ptr, size_t bytes, const char* what);
 
 // Thread-local error message helpers (sp_api.cu).

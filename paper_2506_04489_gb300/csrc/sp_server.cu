@@ -56,6 +56,8 @@ void sleep_until_s(double t)
     }
 }
 
+constexpr double kServerEps = 1e-4;  // GS cutoff of the served plans
+
 size_t io_size(sp_precision p) { return p == SP_FP32 ? 4 : 8; }
 
 struct Req {
@@ -116,18 +118,19 @@ struct sp_server_s {
 namespace {
 using Srv = sp_server_s;
 
+// Everything a resident plan and its batch buffers hold; 1 MiB more for the allocations'
+// rounding.  Sizes that no plan takes count what their 2n passes would need at least, so
+// that they fail where the plan is refused.
 size_t entry_bytes(const Srv* s, int n, sp_precision p)
 {
-    const size_t c = (p == SP_FP64 || p == SP_DF32) ? 16 : 8, r = io_size(p);
-    const size_t ldz = (size_t)(n + 1 + 7) / 8 * 8, nn = (size_t)n;
-    const int N[3] = {2 * n, 2 * n, 2 * n};
-    int F[3];
-    const size_t f = sp_embeds(N, p, F) ? (size_t)F[0] : 2 * nn;  // transform length of the passes
-    const size_t ldf = (f / 2 + 1 + 7) / 8 * 8;
-    const size_t work = (size_t)s->cfg.max_batch * c * nn * f * ldf;
-    const size_t tables = (nn + 1) * (nn + 1) * ldz * 8 + (f / 2 + 1) * (f / 2 + 1) * ldf * (p == SP_DF32 ? 8 : 4) + 3 * 2 * nn * 32;
-    const size_t io = 2 * (size_t)s->cfg.max_batch * nn * nn * nn * r;
-    return work + tables + io + (1u << 20);
+    const size_t io = 2 * (size_t)s->cfg.max_batch * n * n * n * io_size(p), slack = 1u << 20;
+    if (n < 2 || n > 1024) {
+        const size_t c = (p == SP_FP64 || p == SP_DF32) ? 16 : 8, nn = (size_t)n, ldz = (nn + 1 + 7) / 8 * 8;
+        return (size_t)s->cfg.max_batch * c * nn * 2 * nn * ldz + (nn + 1) * (nn + 1) * ldz * (8 + c / 2) + io + slack;
+    }
+    const int nn[3] = {n, n, n};
+    const double lo[3] = {s->cfg.lo, s->cfg.lo, s->cfg.lo}, hi[3] = {s->cfg.hi, s->cfg.hi, s->cfg.hi};
+    return sp_plan_bytes(nn, lo, hi, kServerEps, p, s->cfg.max_batch, true) + io + slack;
 }
 
 int batch_cap(const Srv* s, int n)
@@ -207,7 +210,7 @@ Entry* get_entry(Srv* s, Key key, sp_status* err)
     e->prec = prec;
     const int nn[3] = {n, n, n};
     const double lo[3] = {s->cfg.lo, s->cfg.lo, s->cfg.lo}, hi[3] = {s->cfg.hi, s->cfg.hi, s->cfg.hi};
-    sp_status rc = sp_plan_create(&e->plan, nn, lo, hi, 2, nullptr, nullptr, 0, 1e-4, prec, s->cfg.max_batch);
+    sp_status rc = sp_plan_create(&e->plan, nn, lo, hi, 2, nullptr, nullptr, 0, kServerEps, prec, s->cfg.max_batch);
     if (rc == SP_OK) rc = sp_kernel_precompute(e->plan, s->mem_st);
     const size_t io = (size_t)s->cfg.max_batch * (size_t)n * n * n * io_size(prec);
     if (rc == SP_OK) rc = sp_cuda_check(cudaMallocAsync(&e->d_in, io, s->mem_st), "server batch buffer");

@@ -46,38 +46,64 @@ F_LENGTHS = (16, 32, 48, 64, 72, 80, 96, 128, 144, 160, 192, 200, 216, 256, 288,
              768, 864, 1024, 1280, 1536, 2048)
 
 
+TWIDDLE_ROOM = 8192  # entries reserved per axis for the staged twiddles
+NOALLOC_BYTES = 64 << 20  # static scratch of sp_solve_noalloc
+
+
+def _bluestein(N: int) -> bool:
+    for p in (2, 3, 5, 7):
+        while N % p == 0:
+            N //= p
+    return N != 1
+
+
 def transform_length(n: int, precision: str) -> int:
-    """Transform length per axis of the solve passes of an n^3 grid (the library's rule)."""
+    """Transform length per axis of the solve passes of an n^3 grid, n <= 1024 (the
+    library's rule)."""
     N = 2 * n
     if N in TUNED_LENGTHS:
         return N
-    F = next((f for f in F_LENGTHS if f >= N), N)  # no plan takes 2n > 2048
-    m = N
-    for p in (2, 3, 5, 7):
-        while m % p == 0:
-            m //= p
+    F = next(f for f in F_LENGTHS if f >= N)
     limit = {"fp64": 1.8, "df32": 2.5}.get(precision, 4.0)
-    if m != 1:
+    if _bluestein(N):
         limit *= 4.0
     elif n <= 32:
         limit = 4.0
     return F if (F / N) ** 3 <= limit else N
 
 
-def entry_bytes(n: int, precision: str, max_batch: int) -> int:
-    """Device bytes of one resident plan of an n^3 grid with batch buffers for max_batch
-    requests: workspace, multiplier octant and its pass-precision copy (on the octant of the
-    passes' transform length), twiddles, and the input and output batch buffers (plus 1 MiB
-    for small tables)."""
+def entry_bytes(n: int, precision: str, max_batch: int, lo: float = -1.0, hi: float = 1.0) -> int:
+    """Device bytes of one resident plan of an n^3 grid on [lo, hi]^3 with batch buffers for
+    max_batch requests: every buffer the plan holds, the input and output batch buffers, and
+    1 MiB for the allocations' rounding (the library's sp_server_entry_bytes)."""
     c = 16 if precision in ("fp64", "df32") else 8
     r = 4 if precision == "fp32" else 8
-    ldz = (n + 1 + 7) // 8 * 8
+    half = {"fp64": 0, "df32": 8}.get(precision, 4)  # pass-precision copy of an FP64 value
+    N, ldz = 2 * n, (n + 1 + 7) // 8 * 8
+    octant = (n + 1) * (n + 1) * ldz
+    io = 2 * max_batch * n ** 3 * r + (1 << 20)
+    if not 2 <= n <= 1024:  # no plan takes these
+        return max_batch * c * n * N * ldz + octant * (8 + c // 2) + io
     f = transform_length(n, precision)
     ldf = (f // 2 + 1 + 7) // 8 * 8
-    work = max_batch * c * n * f * ldf
-    tables = (n + 1) * (n + 1) * ldz * 8 + (f // 2 + 1) ** 2 * ldf * (8 if precision == "df32" else 4) + 3 * 2 * n * 32
-    io = 2 * max_batch * n ** 3 * r
-    return work + tables + io + (1 << 20)
+    # GS table (cutoff 1e-4): status word, weights and exponents, one pair of 1D tables
+    eta, L = 1e-17, n * ((hi - lo) / (n - 1))
+    tau = math.log(eta * math.sqrt(math.pi) / (2.0 * math.sqrt(L * L + L * L + L * L)))
+    terms = math.ceil((math.log(math.sqrt(math.log(1.0 / eta)) / 1e-4) + 0.5 - tau) / 0.1) + 1
+    total = 256 + 16 * terms + 16 * terms * (n + 1) + 8 * octant
+    emb = N not in TUNED_LENGTHS and f in F_LENGTHS  # the passes run on f
+    n_bytes, f_bytes = c * n * N * ldz, c * n * f * ldf
+    if not emb or (n_bytes <= NOALLOC_BYTES < f_bytes):
+        total += half * octant
+    if emb:
+        total += c // 2 * (f // 2 + 1) ** 2 * ldf + 3 * c * (f + TWIDDLE_ROOM)
+    total += 3 * (16 * N + 8 * (N + TWIDDLE_ROOM) + 16 * (N + TWIDDLE_ROOM))
+    if _bluestein(N):
+        M = 1
+        while M < 2 * N - 1:
+            M *= 2
+        total += 3 * c * (N + 3 * M)
+    return total + max_batch * f_bytes + io
 
 
 Done = collections.namedtuple("Done", "arrival done_at key launched_at", defaults=(None,))
