@@ -444,13 +444,35 @@ template <class R> __global__ void k_put_columns(long long rows, int cols, const
 
 inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
-struct DevBuf {  // scratch device allocation freed at scope exit (stream-ordered)
-    void* p = nullptr;
+// Scratch of one step of the precompute, freed at scope exit (stream-ordered).  Where the
+// device has no memory left for it, it lies in the plan's workspace, which no solve uses
+// meanwhile (solves are ordered against the precompute) and which a plan on lengths F >= 2n
+// holds larger: such a plan leaves less memory free than one on 2n, and its change of period
+// wants more (500 x 500 x 20, FP32: 105 MB beside a workspace of 131 MB).
+struct Scratch {
     cudaStream_t st;
-    explicit DevBuf(cudaStream_t s) : st(s) {}
-    cudaError_t alloc(size_t bytes) { return cudaMallocAsync(&p, bytes, st); }
-    ~DevBuf() { if (p) cudaFreeAsync(p, st); }
-    double* d() const { return (double*)p; }
+    unsigned char* room;
+    size_t left;
+    void* own[8];
+    int nown = 0;
+    Scratch(sp_plan p, cudaStream_t s) : st(s), room((unsigned char*)p->d_work), left(p->work_bytes) {}
+    Scratch(const Scratch&) = delete;
+    double* take(long long values)  // NULL: it fits neither
+    {
+        const size_t bytes = (sizeof(double) * (size_t)values + 255) / 256 * 256;
+        void* q = nullptr;
+        if (nown < 8 && cudaMallocAsync(&q, bytes, st) == cudaSuccess) return (double*)(own[nown++] = q);
+        cudaGetLastError();  // allocation failures are not sticky: clear them
+        if (bytes > left) return nullptr;
+        q = room;
+        room += bytes;
+        left -= bytes;
+        return (double*)q;
+    }
+    ~Scratch()
+    {
+        for (int i = 0; i < nown; ++i) cudaFreeAsync(own[i], st);
+    }
 };
 
 }  // namespace
@@ -478,18 +500,16 @@ static sp_status setup_axis(sp_plan p, int ax, cudaStream_t st)
         // over a panel (a L^2 < 40: at most 4.2 more of phase at n = 33)
         const int P = n > 32 ? (n + 2) / 3 : (n > 8 ? n : 8), Q = kGLQ;
         const long long nq = (long long)P * Q;
-        DevBuf nodes(st), E(st), C(st);
         const long long rn = (long long)s_split * nq;
-        if (nodes.alloc(sizeof(double) * 3 * nq) ||
-            E.alloc(sizeof(double) * 4 * rn) || C.alloc(sizeof(double) * nk * nq))
-            return sp_fail(SP_ERR_OOM, "setup: quadrature scratch allocation failed");
-        double *tpos = nodes.d(), *y = nodes.d() + nq, *wq = nodes.d() + 2 * nq;
-        double *E0 = E.d(), *E2 = E0 + rn, *F0 = E2 + rn, *F2 = F0 + rn;
+        Scratch scratch(p, st);
+        double *tpos = scratch.take(3 * nq), *E0 = scratch.take(4 * rn), *C = scratch.take(nk * nq);
+        if (!tpos || !E0 || !C) return sp_fail(SP_ERR_OOM, "setup: quadrature scratch allocation failed");
+        double *y = tpos + nq, *wq = tpos + 2 * nq, *E2 = E0 + rn, *F0 = E2 + rn, *F2 = F0 + rn;
         k_nodes<<<nblk(nq, 256), 256, 0, st>>>(P, L, tpos, y, wq);
         k_gauss_rows<<<nblk(rn, 256), 256, 0, st>>>(s_split, (int)nq, p->d_gs_a, y, wq, E0, E2, F0, F2);
-        k_cos_rows<<<nblk(nk * nq, 256), 256, 0, st>>>(nk, P, Q, tpos, C.d());
+        k_cos_rows<<<nblk(nk * nq, 256), 256, 0, st>>>(nk, P, Q, tpos, C);
         dim3 grid(nblk(nk, kAxC), nblk(s_split, kAxS), 2);
-        k_axis_sums<<<grid, kAxS * kAxC, 0, st>>>(s_split, nk, (int)nq, E0, C.d(), p->d_gs_a, L, p->d_G[ax], p->d_H[ax]);
+        k_axis_sums<<<grid, kAxS * kAxC, 0, st>>>(s_split, nk, (int)nq, E0, C, p->d_gs_a, L, p->d_G[ax], p->d_H[ax]);
         rc = sp_cuda_check(cudaGetLastError(), "setup: 1D integral kernels");
         if (rc) return rc;
     }
@@ -522,51 +542,56 @@ void sp_gs_exponents(const sp_plan p, double* a)
 }
 
 // Multiplier of the solve passes' lengths F from the 2n one (both FP64, rounded to the pass
-// type last): one contraction per axis whose length changes, 64 output columns at a time so
-// that the scratch stays at three slabs of (F0/2 + 1)(F1/2 + 1) x 64.
+// type last): one contraction per axis whose length changes, up to 64 output columns at a time
+// so that the scratch stays at two slabs of (F0/2 + 1)(F1/2 + 1) x 64, fewer where it is short.
 static sp_status setup_period(sp_plan p, cudaStream_t st)
 {
     const int n0p = p->n[0] + 1, n1p = p->n[1] + 1, n2p = p->n[2] + 1;
     const int q0 = p->F[0] / 2 + 1, q1 = p->F[1] / 2 + 1, q2 = p->F[2] / 2 + 1;
-    DevBuf T0(st), T1(st), T2(st), X(st), Y(st);
-    DevBuf* T[3] = {&T0, &T1, &T2};
-    constexpr int CW = 64;
+    Scratch scratch(p, st);
+    double* T[3] = {};
     for (int ax = 0; ax < 3; ++ax) {
         if (p->F[ax] == p->N[ax]) continue;
         const long long cnt = (long long)(p->n[ax] + 1) * (p->F[ax] / 2 + 1);
-        if (T[ax]->alloc(sizeof(double) * cnt)) return sp_fail(SP_ERR_OOM, "setup: period scratch allocation failed");
-        k_period_rows<<<nblk(cnt, 256), 256, 0, st>>>(p->n[ax], p->F[ax], T[ax]->d());
+        if (!(T[ax] = scratch.take(cnt))) return sp_fail(SP_ERR_OOM, "setup: period scratch allocation failed");
+        k_period_rows<<<nblk(cnt, 256), 256, 0, st>>>(p->n[ax], p->F[ax], T[ax]);
     }
-    const size_t slab = sizeof(double) * CW * (size_t)(q0 > n0p ? q0 : n0p) * (q1 > n1p ? q1 : n1p);
-    if (X.alloc(slab) || Y.alloc(slab)) return sp_fail(SP_ERR_OOM, "setup: period scratch allocation failed");
+    const long long column = (long long)(q0 > n0p ? q0 : n0p) * (q1 > n1p ? q1 : n1p);
+    int CW = q2 < 64 ? q2 : 64;
+    double* X;
+    while (!(X = scratch.take(2 * CW * column))) {
+        if (CW == 1) return sp_fail(SP_ERR_OOM, "setup: period scratch allocation failed");
+        CW = CW >= 32 ? CW / 2 / 16 * 16 : CW / 2;  // whole tiles while there are any
+    }
+    double* Y = X + CW * column;
     for (int c0 = 0; c0 < q2; c0 += CW) {
         const int cols = q2 - c0 < CW ? q2 - c0 : CW;
         const double* cur = p->d_M64 + c0;  // [n1p][n0p][cols], row stride ld
         long long ld = p->ldz;
-        double* next = X.d();
-        if (T2.p) {
+        double* next = X;
+        if (T[2]) {
             dim3 grid(nblk((long long)n0p * n1p, TM), nblk(cols, TN));
             k_dgemm_nt<<<grid, kGemmThreads, 0, st>>>(n0p * n1p, cols, n2p, p->d_M64, (long long)p->ldz,
-                                             T2.d() + (long long)c0 * n2p, (long long)n2p, EpiStore{next, CW});
+                                             T[2] + (long long)c0 * n2p, (long long)n2p, EpiStore{next, CW});
             cur = next;
             ld = CW;
-            next = Y.d();
+            next = Y;
         }
-        if (T0.p) {
+        if (T[0]) {
             dim3 grid(nblk(cols, kNnT), nblk(q0, kNnT), n1p);
-            k_dgemm_nn<<<grid, 64, 0, st>>>(q0, cols, n0p, T0.d(), cur, ld, ld * n0p, next, CW, (long long)CW * q0);
+            k_dgemm_nn<<<grid, 64, 0, st>>>(q0, cols, n0p, T[0], cur, ld, ld * n0p, next, CW, (long long)CW * q0);
             cur = next;
             ld = CW;
-            next = cur == X.d() ? Y.d() : X.d();
+            next = cur == X ? Y : X;
         }
-        if (T1.p) {  // rows (k0', column) of one k1 are contiguous, or ld apart without an earlier step
+        if (T[1]) {  // rows (k0', column) of one k1 are contiguous, or ld apart without an earlier step
             const long long w = (long long)q0 * ld;
             if (ld == CW) {
                 dim3 grid(nblk(w, kNnT), nblk(q1, kNnT));
-                k_dgemm_nn<<<grid, 64, 0, st>>>(q1, (int)w, n1p, T1.d(), cur, w, 0, next, w, 0);
+                k_dgemm_nn<<<grid, 64, 0, st>>>(q1, (int)w, n1p, T[1], cur, w, 0, next, w, 0);
             } else {
                 dim3 grid(nblk(cols, kNnT), nblk(q1, kNnT), q0);  // one k0 at a time: batch stride ld
-                k_dgemm_nn<<<grid, 64, 0, st>>>(q1, cols, n1p, T1.d(), cur, w, ld, next, (long long)CW * q0, CW);
+                k_dgemm_nn<<<grid, 64, 0, st>>>(q1, cols, n1p, T[1], cur, w, ld, next, (long long)CW * q0, CW);
                 ld = CW;
             }
             cur = next;
@@ -616,12 +641,8 @@ sp_status sp_setup_run(sp_plan p, cudaStream_t st)
         const int K = plain ? S : 2 * S;  // contraction length (GS columns)
         long long most = (140LL << 20) / (8LL * K);
         most = most < 256 ? 256 : (most > 16384 ? 16384 : most);
-        const int chunks = (int)((rows_total + most - 1) / most);
-        const int chunk = (int)((rows_total + chunks - 1) / chunks);
-        DevBuf Ap(st), B0(st), B1(st), B2(st);
-        DevBuf* B[3] = {&B0, &B1, &B2};
+        Scratch scratch(p, st);
         double* bt[3];
-        if (Ap.alloc(sizeof(double) * (size_t)chunk * K)) return sp_fail(SP_ERR_OOM, "setup: multiplier scratch allocation failed");
         for (int ax = 0; ax < 3; ++ax) {
             int same = ax;
             for (int q = ax - 1; q >= 0; --q)
@@ -631,9 +652,16 @@ sp_status sp_setup_run(sp_plan p, cudaStream_t st)
                 continue;
             }
             const int nk = p->n[ax] + 1;
-            if (B[ax]->alloc(sizeof(double) * (size_t)nk * 2 * S)) return sp_fail(SP_ERR_OOM, "setup: multiplier scratch allocation failed");
-            bt[ax] = B[ax]->d();
+            if (!(bt[ax] = scratch.take((long long)nk * 2 * S))) return sp_fail(SP_ERR_OOM, "setup: multiplier scratch allocation failed");
             k_mult_rhs<<<dim3(nblk(2 * S, 256), nk), 256, 0, st>>>(S, nk, p->d_G[ax], p->d_H[ax], bt[ax]);
+        }
+        int chunk;
+        double* Ap;
+        for (;; most /= 2) {  // halved while it does not fit
+            const int chunks = (int)((rows_total + most - 1) / most);
+            chunk = (int)((rows_total + chunks - 1) / chunks);
+            if ((Ap = scratch.take((long long)chunk * K))) break;
+            if (most <= 16) return sp_fail(SP_ERR_OOM, "setup: multiplier scratch allocation failed");
         }
         EpiMultiplier epi;
         epi.M = p->d_M64;
@@ -649,12 +677,12 @@ sp_status sp_setup_run(sp_plan p, cudaStream_t st)
         for (long long r0 = 0; r0 < rows_total; r0 += chunk) {
             int rows = (int)((rows_total - r0) < chunk ? (rows_total - r0) : chunk);
             if (plain)
-                k_plain_lhs<<<dim3(nblk(S, 256), rows), 256, 0, st>>>((int)r0, S, n0p, sym, p->d_gs_w, bt[0], bt[1], Ap.d());
+                k_plain_lhs<<<dim3(nblk(S, 256), rows), 256, 0, st>>>((int)r0, S, n0p, sym, p->d_gs_w, bt[0], bt[1], Ap);
             else
-                k_mult_lhs<<<dim3(nblk(2 * S, 256), rows), 256, 0, st>>>((int)r0, S, n0p, sym, p->d_gs_w, bt[0], bt[1], Ap.d());
+                k_mult_lhs<<<dim3(nblk(2 * S, 256), rows), 256, 0, st>>>((int)r0, S, n0p, sym, p->d_gs_w, bt[0], bt[1], Ap);
             epi.row0 = (int)r0;
             dim3 grid(nblk(rows, TM), nblk(n2p, TN));
-            k_dgemm_nt<<<grid, kGemmThreads, 0, st>>>(rows, n2p, K, Ap.d(), K, bt[2], 2 * S, epi);
+            k_dgemm_nt<<<grid, kGemmThreads, 0, st>>>(rows, n2p, K, Ap, K, bt[2], 2 * S, epi);
         }
         if (cube) k_cube_fill<<<nblk((long long)n0p * n0p * n0p, 256), 256, 0, st>>>(n0p, p->ldz, p->d_M64);
         const long long mcount = (long long)n0p * n1p * p->ldz;
