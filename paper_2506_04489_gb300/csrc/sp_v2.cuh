@@ -992,6 +992,43 @@ template <class R> sp_status stage_twiddles(sp_plan p, cudaStream_t st)
     return SP_OK;
 }
 
+// Arguments of the passes of a solve of `batch` right-hand sides, as it launches them: the z
+// passes' (rho and u are the caller's to set), the y passes' and the x pass's.
+template <class R> void pass_args(sp_plan p, int batch, ZArgs2& z, LArgs& y, LArgs& x)
+{
+    z = {};
+    z.W = p->d_work;
+    z.n1 = p->n[1];
+    z.n2 = p->n[2];
+    z.lines = (long long)p->n[0] * p->n[1];
+    z.plane = p->plane;
+    z.ldz = p->ldz;
+    z.io_bs = (long long)p->n[0] * p->n[1] * p->n[2];
+    z.w_bs = (long long)p->n[0] * p->plane;
+    z.tw = Tabs<R>::tw(p, 2);
+    z.B = p->tile_z;
+    z.dependent = (size_t)batch * z.w_bs * sizeof(cpx<R>) <= kDependentBytes;
+    y = {};
+    y.in = y.out = p->d_work;
+    y.in_os = y.out_os = p->plane;
+    y.in_es = y.out_es = p->ldz;
+    y.in_bs = y.out_bs = (long long)p->n[0] * p->plane;
+    y.ncol = p->n[2] + 1;
+    y.in_ld = p->ldz;
+    y.tw = Tabs<R>::tw(p, 1);
+    y.B = p->tile_line[1];
+    y.dependent = z.dependent;
+    x = y;
+    x.in_os = x.out_os = p->ldz;
+    x.in_es = x.out_es = p->plane;
+    x.tw = Tabs<R>::tw(p, 0);
+    x.M = Tabs<R>::M(p);
+    x.B = p->tile_line[0];
+    x.No = p->N[1];
+    x.nh_line = p->n[0];
+    x.ldzM = p->ldz;
+}
+
 // The whole solve; `work` is the workspace (the plan's, or another of the same size).
 template <class R, class Tio>
 sp_status solve(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st, bool mark)
@@ -1005,39 +1042,11 @@ sp_status solve(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st,
     p->pass_name[2] = "x_multiply";
     p->pass_name[3] = "y_inverse";
     p->pass_name[4] = "z_inverse";
-    ZArgs2 z = {};
+    ZArgs2 z;
+    LArgs y, x;
+    pass_args<R>(p, batch, z, y, x);
     z.rho = rho;
     z.u = u;
-    z.W = p->d_work;
-    z.n1 = p->n[1];
-    z.n2 = p->n[2];
-    z.lines = (long long)p->n[0] * p->n[1];
-    z.plane = p->plane;
-    z.ldz = p->ldz;
-    z.io_bs = (long long)p->n[0] * p->n[1] * p->n[2];
-    z.w_bs = (long long)p->n[0] * p->plane;
-    z.tw = Tabs<R>::tw(p, 2);
-    z.B = p->tile_z;
-    z.dependent = (size_t)batch * z.w_bs * sizeof(cpx<R>) <= kDependentBytes;
-    LArgs y = {};
-    y.in = y.out = p->d_work;
-    y.in_os = y.out_os = p->plane;
-    y.in_es = y.out_es = p->ldz;
-    y.in_bs = y.out_bs = (long long)p->n[0] * p->plane;
-    y.ncol = p->n[2] + 1;
-    y.in_ld = p->ldz;
-    y.tw = Tabs<R>::tw(p, 1);
-    y.B = p->tile_line[1];
-    y.dependent = z.dependent;
-    LArgs x = y;
-    x.in_os = x.out_os = p->ldz;
-    x.in_es = x.out_es = p->plane;
-    x.tw = Tabs<R>::tw(p, 0);
-    x.M = Tabs<R>::M(p);
-    x.B = p->tile_line[0];
-    x.No = p->N[1];
-    x.nh_line = p->n[0];
-    x.ldzM = p->ldz;
     // Each pass writes its outer indices in increasing order, so what it wrote last is still
     // in L2 when the next pass starts: the y forward pass walks the planes the z forward
     // pass wrote from the last one down, and the z inverse pass the rows the y inverse pass
@@ -1069,36 +1078,13 @@ sp_status solve(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st,
 template <class R, class Tio>
 float time_pass(sp_plan p, int pass, int tile, int batch, int iters, cudaStream_t st, int variant)
 {
-    ZArgs2 z = {};
+    ZArgs2 z;
+    LArgs y, x;
+    pass_args<R>(p, batch, z, y, x);
     z.rho = p->d_work;
     z.u = (char*)p->d_work + p->work_bytes / 2;  // the z passes only need valid addresses
-    z.W = p->d_work;
-    z.n1 = p->n[1];
-    z.n2 = p->n[2];
-    z.lines = (long long)p->n[0] * p->n[1];
-    z.plane = p->plane;
-    z.ldz = p->ldz;
     z.io_bs = 0;
-    z.w_bs = (long long)p->n[0] * p->plane;
-    z.tw = Tabs<R>::tw(p, 2);
-    z.B = tile;
-    LArgs y = {};
-    y.in = y.out = p->d_work;
-    y.in_os = y.out_os = p->plane;
-    y.in_es = y.out_es = p->ldz;
-    y.in_bs = y.out_bs = (long long)p->n[0] * p->plane;
-    y.ncol = p->n[2] + 1;
-    y.in_ld = p->ldz;
-    y.tw = Tabs<R>::tw(p, 1);
-    y.B = tile;
-    LArgs x = y;
-    x.in_os = x.out_os = p->ldz;
-    x.in_es = x.out_es = p->plane;
-    x.tw = Tabs<R>::tw(p, 0);
-    x.M = Tabs<R>::M(p);
-    x.No = p->N[1];
-    x.nh_line = p->n[0];
-    x.ldzM = p->ldz;
+    z.B = y.B = x.B = tile;
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess) return -1.f;
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return -1.f; }
