@@ -415,7 +415,8 @@ sp_status sp_solve_noalloc(const sp_plan plan, const void* rho, void* u, sp_stre
  *     workspace and batch buffers stay on the device), created on first use, or in
  *     advance by sp_server_prepare, within budget_bytes of device memory (estimate:
  *     sp_server_entry_bytes); idle plans of other keys are evicted, least recently used
- *     first, to make room; a request waits while its key's plans are busy;
+ *     first, to make room, and a plan whose longer transforms (sp_plan_create) do not fit
+ *     even so runs on 2n where those do; a request waits while its key's plans are busy;
  *   - the key whose oldest request has waited longest is served first; its waiting
  *     requests form one batch (at most max_batch requests, at most max_batch_points grid
  *     points, at least one request);
@@ -479,7 +480,9 @@ sp_status sp_server_shutdown(sp_server srv);
 /* Shut down and free everything the server holds.  No call on srv may be in progress or
  * follow. */
 sp_status sp_server_destroy(sp_server srv);
-/* Device bytes the server counts against its budget for one resident plan of the key. */
+/* Device bytes the server counts against its budget for one resident plan of the key (on the
+ * longer transforms of sp_plan_create where the size takes them; a plan the server puts on 2n
+ * for want of room counts less). */
 size_t sp_server_entry_bytes(const sp_server_config* cfg, int n, sp_precision prec);
 /* The server's clock: seconds on the host's monotonic clock. */
 double sp_monotonic_seconds(void);

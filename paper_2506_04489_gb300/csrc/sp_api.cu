@@ -158,6 +158,12 @@ extern "C" sp_status sp_plan_create_ex(sp_plan* out, const int n[3], const doubl
     return create_plan(out, n, box_lo, box_hi, padding, gs_w, gs_a, gs_terms, eps, prec, max_batch, allocator, false);
 }
 
+sp_status sp_plan_create_2n(sp_plan* out, const int n[3], const double box_lo[3], const double box_hi[3], double eps,
+                            sp_precision prec, int max_batch)
+{
+    return create_plan(out, n, box_lo, box_hi, 2, nullptr, nullptr, 0, eps, prec, max_batch, nullptr, false);
+}
+
 // What the sizes of a plan's buffers depend on: lengths, strides and the GS table's length
 // (0 gs_terms: generated).  Host only.
 static void plan_geometry(sp_plan p, const int n[3], const double box_lo[3], const double box_hi[3], int gs_terms,

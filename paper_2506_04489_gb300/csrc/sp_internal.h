@@ -133,6 +133,9 @@ void sp_bluestein_fill(const sp_plan_s* p, int ax, void* host);
 // buffers, on the lengths F where sp_embeds says so and may_embed, else on 2n.
 size_t sp_plan_bytes(const int n[3], const double box_lo[3], const double box_hi[3], double eps, sp_precision prec,
                      int max_batch, bool may_embed);
+// sp_plan_create with a generated GS table and the passes on 2n, whatever sp_embeds says.
+sp_status sp_plan_create_2n(sp_plan* out, const int n[3], const double box_lo[3], const double box_hi[3], double eps,
+                            sp_precision prec, int max_batch);
 // Device allocation owned by the plan (the caller's allocator, else cudaMallocAsync).
 sp_status sp_plan_alloc(sp_plan p, void** ptr, size_t bytes, const char* what);
 

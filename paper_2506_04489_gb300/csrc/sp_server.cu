@@ -120,8 +120,9 @@ using Srv = sp_server_s;
 
 // Everything a resident plan and its batch buffers hold; 1 MiB more for the allocations'
 // rounding.  Sizes that no plan takes count what their 2n passes would need at least, so
-// that they fail where the plan is refused.
-size_t entry_bytes(const Srv* s, int n, sp_precision p)
+// that they fail where the plan is refused.  longer: on lengths F >= 2n where the size takes
+// them; otherwise on 2n.
+size_t entry_bytes(const Srv* s, int n, sp_precision p, bool longer)
 {
     const size_t io = 2 * (size_t)s->cfg.max_batch * n * n * n * io_size(p), slack = 1u << 20;
     if (n < 2 || n > 1024) {
@@ -130,7 +131,13 @@ size_t entry_bytes(const Srv* s, int n, sp_precision p)
     }
     const int nn[3] = {n, n, n};
     const double lo[3] = {s->cfg.lo, s->cfg.lo, s->cfg.lo}, hi[3] = {s->cfg.hi, s->cfg.hi, s->cfg.hi};
-    return sp_plan_bytes(nn, lo, hi, kServerEps, p, s->cfg.max_batch, true) + io + slack;
+    return sp_plan_bytes(nn, lo, hi, kServerEps, p, s->cfg.max_batch, longer) + io + slack;
+}
+
+// The smaller of the two: what a key needs to be served at all.
+size_t least_bytes(const Srv* s, int n, sp_precision p)
+{
+    return std::min(entry_bytes(s, n, p, true), entry_bytes(s, n, p, false));
 }
 
 int batch_cap(const Srv* s, int n)
@@ -167,14 +174,20 @@ void destroy_entry(Srv* s, Entry* e)
     delete e;
 }
 
-// Free idle plans of other keys, least recently used first, until `need` fits.
+// Free idle plans of other keys, least recently used first, until `need` fits; none if it
+// would not fit without all of them.
 bool evict_for(Srv* s, size_t need, Key keep)
 {
     std::vector<std::pair<double, Entry*>> idle;
+    double held = s->used_bytes;
     for (auto& kv : s->entries)
         if (kv.first != keep)
             for (Entry* e : kv.second)
-                if (!e->busy) idle.emplace_back(e->last_used, e);
+                if (!e->busy) {
+                    idle.emplace_back(e->last_used, e);
+                    held -= (double)e->bytes;
+                }
+    if (held + (double)need > s->cfg.budget_bytes) return false;
     std::sort(idle.begin(), idle.end(), [](const std::pair<double, Entry*>& a, const std::pair<double, Entry*>& b) {
         return a.first < b.first;
     });
@@ -185,12 +198,13 @@ bool evict_for(Srv* s, size_t need, Key keep)
         lst.erase(std::find(lst.begin(), lst.end(), e));
         destroy_entry(s, e);
     }
-    return s->used_bytes + (double)need <= s->cfg.budget_bytes;
+    return true;
 }
 
 // A free resident plan of the key, a new one within the budget, or NULL (wait).  On a
-// failure to create one, *err is set.
-Entry* get_entry(Srv* s, Key key, sp_status* err)
+// failure to create one, *err is set.  A size whose passes run longer transforms takes them
+// while they fit the budget, and 2n where only those do.
+Entry* get_entry(Srv* s, Key key, sp_status* err, bool may_evict = true)
 {
     *err = SP_OK;
     auto& lst = s->entries[key];
@@ -199,8 +213,16 @@ Entry* get_entry(Srv* s, Key key, sp_status* err)
     if ((int)lst.size() >= s->cfg.plans_per_key) return nullptr;
     const int n = key.first;
     const sp_precision prec = (sp_precision)key.second;
-    const size_t need = entry_bytes(s, n, prec);
-    if (s->used_bytes + (double)need > s->cfg.budget_bytes && !evict_for(s, need, key)) return nullptr;
+    const auto fits = [&](size_t need) {
+        return s->used_bytes + (double)need <= s->cfg.budget_bytes || (may_evict && evict_for(s, need, key));
+    };
+    bool longer = true;
+    size_t need = entry_bytes(s, n, prec, true);
+    if (!fits(need)) {
+        longer = false;
+        need = entry_bytes(s, n, prec, false);
+        if (!fits(need)) return nullptr;
+    }
     Entry* e = new (std::nothrow) Entry();
     if (!e) {
         *err = SP_ERR_OOM;
@@ -210,7 +232,8 @@ Entry* get_entry(Srv* s, Key key, sp_status* err)
     e->prec = prec;
     const int nn[3] = {n, n, n};
     const double lo[3] = {s->cfg.lo, s->cfg.lo, s->cfg.lo}, hi[3] = {s->cfg.hi, s->cfg.hi, s->cfg.hi};
-    sp_status rc = sp_plan_create(&e->plan, nn, lo, hi, 2, nullptr, nullptr, 0, kServerEps, prec, s->cfg.max_batch);
+    sp_status rc = longer ? sp_plan_create(&e->plan, nn, lo, hi, 2, nullptr, nullptr, 0, kServerEps, prec, s->cfg.max_batch)
+                          : sp_plan_create_2n(&e->plan, nn, lo, hi, kServerEps, prec, s->cfg.max_batch);
     if (rc == SP_OK) rc = sp_kernel_precompute(e->plan, s->mem_st);
     const size_t io = (size_t)s->cfg.max_batch * (size_t)n * n * n * io_size(prec);
     if (rc == SP_OK) rc = sp_cuda_check(cudaMallocAsync(&e->d_in, io, s->mem_st), "server batch buffer");
@@ -318,7 +341,7 @@ bool schedule_one(Srv* s)
         const Key key = k.second;
         auto& q = s->pending[key];
         const sp_precision prec = (sp_precision)key.second;
-        if ((double)entry_bytes(s, key.first, prec) > s->cfg.budget_bytes) {  // can never be admitted
+        if ((double)least_bytes(s, key.first, prec) > s->cfg.budget_bytes) {  // can never be admitted
             const double t = now_s();
             while (!q.empty()) {
                 finish(s, q.front(), SP_ERR_OOM, t);
@@ -406,7 +429,7 @@ extern "C" size_t sp_server_entry_bytes(const sp_server_config* cfg, int n, sp_p
     if (!cfg || n < 1) return 0;
     Srv tmp;
     tmp.cfg = *cfg;
-    return entry_bytes(&tmp, n, prec);
+    return entry_bytes(&tmp, n, prec, true);
 }
 
 extern "C" sp_status sp_server_create(sp_server* out, const sp_server_config* cfg)
@@ -472,9 +495,9 @@ extern "C" sp_status sp_server_prepare(sp_server s, int n, sp_precision prec)
     }
     sp_status rc = SP_OK;
     while ((int)lst.size() < s->cfg.plans_per_key &&
-           s->used_bytes + (double)entry_bytes(s, n, prec) <= s->cfg.budget_bytes) {
+           s->used_bytes + (double)least_bytes(s, n, prec) <= s->cfg.budget_bytes) {
         sp_status err;
-        Entry* e = get_entry(s, key, &err);
+        Entry* e = get_entry(s, key, &err, false);
         if (!e) {
             rc = err != SP_OK ? err : sp_fail(SP_ERR_OOM, "no room for another plan");
             break;
