@@ -111,14 +111,48 @@ int sp_f_length(int N)
     return 0;
 }
 
+// Time of an FP64 solve of `batch` right-hand sides on lengths F over that on 2n, from a fit to
+// 706 measured solves (2 to 1000 points an axis, batches up to 15000; standard deviation 14 % on
+// F, 23 % on 2n): launches and latency (us), then the columns that the tiles hold, empty ones
+// included, times their length and a cost an element (ps): by stages on 2n, by the transform's
+// operations on F.
+static double fp64_longer_ratio(const int N[3], const int F[3], int batch)
+{
+    const auto up = [](long long a, int b) { return (double)((a + b - 1) / b * b); };
+    const long long n0 = N[0] / 2, n1 = N[1] / 2, n2 = N[2] / 2;
+    double longer = 0.0, own = 0.0;
+    for (int ax = 0; ax < 3; ++ax) {
+        RadixPlan rp;
+        const bool blue = !sp_radix_plan(N[ax], &rp);
+        int rows = N[ax];
+        if (blue) {
+            for (rows = 1; rows < 2 * N[ax] - 1;) rows *= 2;
+            sp_radix_plan(rows, &rp);
+        }
+        const int tile = sp_line_tile(rows, sizeof(cpx<double>)), tileF = F[ax] <= 48 ? 16 : (F[ax] < 216 ? 8 : 4);
+        const long long outer = ax == 1 ? n0 : N[1], outerF = ax == 1 ? n0 : F[1];
+        const double lines = ax == 2 ? 2 * up((n0 * n1 + 1) / 2, tile) : 2 * outer * up(n2 + 1, tile);
+        const double linesF = ax == 2 ? (double)(n0 * n1) : 2 * outerF * up(F[2] / 2 + 1, tileF);
+        own += lines * (rows * (1.8 + 17.3 * rp.nst) * (blue ? 2.56 : 1.0) + (ax == 2 ? 183.0 * N[2] : 0.0));
+        longer += linesF * F[ax] * 5.23 * log2((double)F[ax]);
+    }
+    return (34.0 + 1e-6 * batch * longer) / (90.0 + 1e-6 * batch * own);
+}
+
 // A grid takes the lengths F unless every padded length has its tuned plan, or the padding to
-// F costs more than the register engine gains over the runtime-radix passes.  That matters
-// only for flat grids, whose short axes round up by up to 8 times.  Gains at equal work:
-// about 2 in FP64 (pipe-bound in both), 2.5 in double-float, 4 and more in FP32, four times
-// that where an axis needs Bluestein's algorithm (512x512x3, growth 2.7: FP64 0.53, double-
-// float 0.96, FP32 1.73 times the speed; 129^3: 11, 12 and 18 times).  Grids of up to 32^3
-// points are bound by latency and gain at any growth measured (7x9x5, growth 3.3: 1.3-1.6).
-bool sp_embeds(const int N[3], sp_precision prec, int F[3])
+// F costs more than the register engine gains over the runtime-radix passes: flat grids, whose
+// short axes round up by up to 8 times, and FP64 cubes with 2n from 98 to 106 (F = 128).  Gains
+// at equal work: about 2 in FP64 (pipe-bound in both), 2.5 in double-float, 4 and more in FP32,
+// four times that where an axis needs Bluestein's algorithm (512x512x3, growth 2.7: FP64 0.53,
+// double-float 0.96, FP32 1.73 times the speed; 129^3: 11, 12 and 18 times).  Grids of up to
+// 32^3 points are bound by latency and gain at any growth measured (7x9x5, growth 3.3: 1.3-1.6).
+// In FP64, bound by its pipe in both engines, what the padding adds is paid in full once a batch
+// fills the chip, and by grids with one Bluestein axis that holds little of the work: there the
+// measured times decide.  Of 706 solves 32 had become slower (100x2x11, batch 909, 3.81 -> 8.67
+// ms; 20x4x10, batch 2500, 2.45 -> 4.58; 784x2x436 1.43 -> 2.53); at a predicted 0.83 none does,
+// and 34 give up gains of up to 41 %, 19 % in the median.  In double-float and FP32 none of 1423
+// solves was slower on F.
+bool sp_embeds(const int N[3], sp_precision prec, int max_batch, int F[3])
 {
     bool tuned = true, blue = false;
     double growth = 1.0;
@@ -135,7 +169,7 @@ bool sp_embeds(const int N[3], sp_precision prec, int F[3])
     double limit = prec == SP_FP64 ? 1.8 : (prec == SP_DF32 ? 2.5 : 4.0);
     if (blue) limit *= 4.0;
     else if (small) limit = 4.0;
-    return !tuned && growth <= limit;
+    return !tuned && growth <= limit && (prec != SP_FP64 || fp64_longer_ratio(N, F, max_batch) <= 0.83);
 }
 
 static sp_status create_plan(sp_plan* out, const int n[3], const double box_lo[3],
@@ -154,7 +188,7 @@ extern "C" sp_status sp_plan_create_ex(sp_plan* out, const int n[3], const doubl
     if (rc != SP_ERR_OOM) return rc;
     int N[3], F[3];
     for (int ax = 0; ax < 3; ++ax) N[ax] = 2 * n[ax];
-    if (!sp_embeds(N, prec, F)) return rc;
+    if (!sp_embeds(N, prec, max_batch, F)) return rc;
     return create_plan(out, n, box_lo, box_hi, padding, gs_w, gs_a, gs_terms, eps, prec, max_batch, allocator, false);
 }
 
@@ -191,7 +225,7 @@ static void plan_geometry(sp_plan p, const int n[3], const double box_lo[3], con
     p->ldz = (n[2] + 1 + 7) & ~7;
     p->plane = 2LL * n[1] * p->ldz;
     const size_t csize = (prec == SP_FP64 || prec == SP_DF32) ? 16 : 8;
-    p->emb = sp_embeds(p->N, prec, p->F) && may_embed;
+    p->emb = sp_embeds(p->N, prec, max_batch, p->F) && may_embed;
     if (!p->emb)
         for (int ax = 0; ax < 3; ++ax) p->F[ax] = p->N[ax];
     p->ldf = (p->F[2] / 2 + 1 + 7) & ~7;

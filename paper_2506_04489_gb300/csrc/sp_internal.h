@@ -162,9 +162,11 @@ sp_status sp_v2_forward_f64(sp_plan p, const void* rho, void* spec, cudaStream_t
 sp_status sp_v2_forward_df(sp_plan p, const void* rho, void* spec, cudaStream_t st);
 bool sp_v2_supported(int N);
 // Shortest transform length of the solve passes for a padded length N <= 2048 (N itself
-// where it has a tuned plan), and whether a grid with these padded lengths takes them.
+// where it has a tuned plan), and whether a plan with these padded lengths takes them.
 int sp_f_length(int N);
-bool sp_embeds(const int N[3], sp_precision prec, int F[3]);
+bool sp_embeds(const int N[3], sp_precision prec, int max_batch, int F[3]);
+// Columns (or pairs of real lines) of a CTA of the 2n passes, `rows` elements of csize bytes each.
+int sp_line_tile(int rows, size_t csize);
 sp_status sp_embed_solve_f32(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st, bool mixed);
 sp_status sp_embed_solve_f64(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st);
 sp_status sp_embed_solve_df(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st);

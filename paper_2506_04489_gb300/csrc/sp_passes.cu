@@ -269,13 +269,6 @@ __global__ void __launch_bounds__(kThreads) k_z_inverse(ZArgs a)
     }
 }
 
-int pick_B(int N, size_t csize)
-{
-    int B = 16;
-    while (B > 1 && 2 * (size_t)N * B * csize > (size_t)kSmemTarget) B /= 2;
-    return B;
-}
-
 template <class K>
 sp_status set_smem(K kernel, size_t bytes)
 {
@@ -329,7 +322,7 @@ sp_status z_pass(sp_plan p, const void* rho, void* u, int batch, bool forward, c
     a.rp = p->rp[2];
     a.tw = tw_of<R>(p, 2);
     a.blue = blue_of(p, 2);
-    a.B = pick_B(line_rows(a.N, a.blue), sizeof(cpx<R>));
+    a.B = sp_line_tile(line_rows(a.N, a.blue), sizeof(cpx<R>));
     const long long pairs = (a.lines + 1) / 2;
     dim3 grid((unsigned)((pairs + a.B - 1) / a.B), (unsigned)batch);
     size_t smem = 2 * (size_t)line_rows(a.N, a.blue) * a.B * sizeof(cpx<R>);
@@ -348,7 +341,7 @@ template <class R>
 sp_status line_pass(const LineArgs& a0, int outer, int batch, cudaStream_t st, const char* what)
 {
     LineArgs a = a0;
-    a.B = pick_B(line_rows(a.N, a.blue), sizeof(cpx<R>));
+    a.B = sp_line_tile(line_rows(a.N, a.blue), sizeof(cpx<R>));
     size_t smem = 2 * (size_t)line_rows(a.N, a.blue) * a.B * sizeof(cpx<R>);
     sp_status rc;
     if ((rc = set_smem(k_lines<R>, smem))) return rc;
@@ -444,6 +437,13 @@ sp_status forward_t(sp_plan p, const void* rho, void* spec, cudaStream_t st)
 bool sp_v2_supported(int N)
 {
     return N == 64 || N == 128 || N == 192 || N == 256 || N == 384 || N == 512 || N == 1024;
+}
+
+int sp_line_tile(int rows, size_t csize)
+{
+    int B = 16;
+    while (B > 1 && 2 * (size_t)rows * B * csize > (size_t)kSmemTarget) B /= 2;
+    return B;
 }
 
 sp_status sp_run_solve(sp_plan p, const void* rho, void* u, int batch, cudaStream_t st)

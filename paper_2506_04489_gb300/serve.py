@@ -57,19 +57,63 @@ def _bluestein(N: int) -> bool:
     return N != 1
 
 
-def transform_length(n: int, precision: str) -> int:
-    """Transform length per axis of the solve passes of an n^3 grid, n <= 1024 (the
-    library's rule)."""
+def _stages(N: int) -> int:
+    """Stages of a 2n transform: radix 8, 4 or 2, then one for each 3, 5 and 7."""
+    twos = (N & -N).bit_length() - 1
+    N >>= twos
+    st = (twos + 2) // 3
+    for p in (3, 5, 7):
+        while N % p == 0:
+            N //= p
+            st += 1
+    return st
+
+
+def _fp64_longer_ratio(n: int, F: int, batch: int) -> float:
+    """Predicted time of an FP64 solve of an n^3 grid on lengths F over that on 2n (the
+    library's fit to measured solves)."""
+    def up(a, b):
+        return float((a + b - 1) // b * b)
+
+    N = rows = 2 * n
+    blue = _bluestein(N)
+    if blue:
+        rows = 1
+        while rows < 2 * N - 1:
+            rows *= 2
+    tile = 16
+    while tile > 1 and 2 * rows * tile * 16 > 64 * 1024:
+        tile //= 2
+    tile_f = 16 if F <= 48 else (8 if F < 216 else 4)
+    own = longer = 0.0
+    for ax in range(3):
+        lines = 2 * up((n * n + 1) // 2, tile) if ax == 2 else 2 * (n if ax == 1 else N) * up(n + 1, tile)
+        lines_f = float(n * n) if ax == 2 else 2 * (n if ax == 1 else F) * up(F // 2 + 1, tile_f)
+        own += lines * (rows * (1.8 + 17.3 * _stages(rows)) * (2.56 if blue else 1.0) + (183.0 * N if ax == 2 else 0.0))
+        longer += lines_f * F * 5.23 * math.log2(F)
+    return (34.0 + 1e-6 * batch * longer) / (90.0 + 1e-6 * batch * own)
+
+
+def _longer(n: int, precision: str, max_batch: int):
+    """The length F >= 2n that the passes of an n^3 grid run on (the library's rule), or None
+    where they run on 2n."""
     N = 2 * n
     if N in TUNED_LENGTHS:
-        return N
+        return None
     F = next(f for f in F_LENGTHS if f >= N)
     limit = {"fp64": 1.8, "df32": 2.5}.get(precision, 4.0)
     if _bluestein(N):
         limit *= 4.0
     elif n <= 32:
         limit = 4.0
-    return F if (F / N) ** 3 <= limit else N
+    if (F / N) ** 3 > limit or (precision == "fp64" and _fp64_longer_ratio(n, F, max_batch) > 0.83):
+        return None
+    return F
+
+
+def transform_length(n: int, precision: str, max_batch: int = 1) -> int:
+    """Transform length per axis of the solve passes of an n^3 grid, n <= 1024."""
+    return _longer(n, precision, max_batch) or 2 * n
 
 
 def entry_bytes(n: int, precision: str, max_batch: int, lo: float = -1.0, hi: float = 1.0) -> int:
@@ -84,18 +128,18 @@ def entry_bytes(n: int, precision: str, max_batch: int, lo: float = -1.0, hi: fl
     io = 2 * max_batch * n ** 3 * r + (1 << 20)
     if not 2 <= n <= 1024:  # no plan takes these
         return max_batch * c * n * N * ldz + octant * (8 + c // 2) + io
-    f = transform_length(n, precision)
+    longer = _longer(n, precision, max_batch)
+    f = longer or N
     ldf = (f // 2 + 1 + 7) // 8 * 8
     # GS table (cutoff 1e-4): status word, weights and exponents, one pair of 1D tables
     eta, L = 1e-17, n * ((hi - lo) / (n - 1))
     tau = math.log(eta * math.sqrt(math.pi) / (2.0 * math.sqrt(L * L + L * L + L * L)))
     terms = math.ceil((math.log(math.sqrt(math.log(1.0 / eta)) / 1e-4) + 0.5 - tau) / 0.1) + 1
     total = 256 + 16 * terms + 16 * terms * (n + 1) + 8 * octant
-    emb = N not in TUNED_LENGTHS and f in F_LENGTHS  # the passes run on f
     n_bytes, f_bytes = c * n * N * ldz, c * n * f * ldf
-    if not emb or (n_bytes <= NOALLOC_BYTES < f_bytes):
+    if not longer or (n_bytes <= NOALLOC_BYTES < f_bytes):
         total += half * octant
-    if emb:
+    if longer:
         total += c // 2 * (f // 2 + 1) ** 2 * ldf + 3 * c * (f + TWIDDLE_ROOM)
     total += 3 * (16 * N + 8 * (N + TWIDDLE_ROOM) + 16 * (N + TWIDDLE_ROOM))
     if _bluestein(N):

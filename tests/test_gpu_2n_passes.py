@@ -104,6 +104,26 @@ def test_flat_grids_run_2n(oracle, n, precision):
     _check_entry_points(plan, oracle)
 
 
+# FP64 pays for padding in full once a batch fills the chip, and where the one Bluestein axis
+# holds little of the work; measured on F against 2n: 1.8, 1.7, 1.5, 1.2, 1.2, 1.1 and 1.8 times
+# the time; then 0.69, 0.90 and 0.67, a growth of 2.1, and a growth of 1
+@pytest.mark.parametrize("n,nb,longer", [((100, 2, 11), 45, False), ((20, 4, 10), 125, False), ((98, 9, 9), 12, False),
+                                         ((12, 12, 12), 128, False), ((14, 14, 14), 128, False), ((21, 18, 9), 29, False),
+                                         ((784, 2, 436), 1, False), ((18, 18, 18), 1, True), ((25, 25, 25), 27, True),
+                                         ((18, 50, 24), 200, True), ((50, 50, 50), 1, False), ((16, 48, 80), 4, True)])
+def test_fp64_runs_the_faster_length(n, nb, longer):
+    plan = Plan(n, LO, HI, precision="fp64", max_batch=nb, precompute=False)
+    assert _runs_2n(plan) != longer
+    plan.close()
+
+
+@pytest.mark.parametrize("n,nb", [((20, 4, 10), 125), ((98, 9, 9), 12), ((12, 12, 12), 128)])
+def test_fp64_batches_on_2n(oracle, n, nb):
+    plan = Plan(n, LO, HI, precision="fp64", max_batch=nb)
+    assert _runs_2n(plan)
+    _check_entry_points(plan, oracle)
+
+
 # the longest lengths (2048 by radix stages, 2042 by Bluestein's algorithm with M = 4096): a
 # density shifted by one cell has the potential shifted by one cell; two solves are compared,
 # each held to the parity tolerance
