@@ -88,14 +88,15 @@ typedef void* sp_stream; /* a cudaStream_t */
  * current device, stream-ordered from its default memory pool (cudaMallocAsync on a stream
  * of the plan's own, complete when this call returns); sp_plan_create_ex takes a caller's
  * allocator.
- * Every precision takes the same lengths.  Where every 2n has a tuned plan (64, 128, 192,
+ * Every precision takes every length.  Where every 2n has a tuned plan (64, 128, 192,
  * 256, 384, 512, 1024), F = 2n.  On other grids the solve passes run on the shortest
- * lengths F >= 2n they are compiled for (4 to 29 % longer in the mean and at most, from 64
- * up): the same aperiodic convolution, its multiplier carried to period F at precompute, so
+ * lengths F >= 2n they are compiled for (for n = 32 to 1024 10 % longer in the mean and 33 % at
+ * most): the same aperiodic convolution, its multiplier carried to period F at precompute, so
  * the results differ from the 2n transforms by rounding only.  The 2n transforms themselves
- * (radix 2..8, 3, 5 and 7 stages, or Bluestein's algorithm) serve sp_forward_spectrum, flat
- * grids whose short axes would round up too far, and a plan whose larger workspace does not
- * fit the device.  Bluestein axes also hold a table of 2n + 3M complex values built on the
+ * (radix 2..8, 3, 5 and 7 stages, or Bluestein's algorithm) serve sp_forward_spectrum, grids
+ * that would round up too far (flat ones, a few cubes), SP_FP64 plans predicted faster on them
+ * (small grids with a large max_batch), and a plan whose larger workspace does not fit the
+ * device.  Bluestein axes also hold a table of 2n + 3M complex values built on the
  * host and copied here.
  */
 sp_status sp_plan_create(sp_plan* out, const int n[3], const double box_lo[3],
@@ -294,7 +295,8 @@ int sp_plan_pass_times(sp_plan plan, double* total_ms, int* launches, const char
  *   rounds differently, so results then agree to the precision's tolerance, not bitwise.
  *   FP32 and mixed plans where the fused plane passes exist then time whole solves of
  *   both schedules and keep the faster (see sp_plan_launch_config).
- *   A no-op for grids without compiled register-resident passes.
+ *   Tunes grids whose 2n all have a tuned plan (sp_plan_create); on other grids it changes
+ *   nothing and returns SP_OK: their passes take tiles by rule, whatever is stored here.
  * sp_plan_tiles -- the tiles in use: line_tiles[3] (columns per CTA of the y and x line
  *   passes, by axis; 0 = default) and *z_tile (pairs of real lines per CTA of the z
  *   passes).  Either pointer may be NULL.
@@ -392,8 +394,7 @@ sp_status sp_graph_destroy(sp_graph graph);
  * else 8) x
  * n0 x F1 x round_up(F2/2 + 1, 8) (F: the passes' transform lengths, sp_plan_create; the
  * 2n passes run where only theirs fits), exceeds it is rejected with SP_ERR_UNSUPPORTED_SIZE
- * (of the supported cube sizes, FP64 fits up to n = 126, double-float up to n = 96, its
- * largest supported length below that, and FP32/mixed up to n = 150).
+ * (cubes fit up to n = 127 in SP_FP64 and SP_DF32, up to n = 159 in SP_FP32 and SP_MIXED).
  * The first call on a device looks up the array's device address (once per device,
  * with that device current) and keeps it for the life of the process; make that first
  * call before any stream capture, and do not use this entry point after

@@ -141,7 +141,8 @@ static double fp64_longer_ratio(const int N[3], const int F[3], int batch)
 
 // A grid takes the lengths F unless every padded length has its tuned plan, or the padding to
 // F costs more than the register engine gains over the runtime-radix passes: flat grids, whose
-// short axes round up by up to 8 times, and FP64 cubes with 2n from 98 to 106 (F = 128).  Gains
+// short axes round up by up to 8 times, and a few cubes (2 to 5, 9 and 10 points an axis in every
+// type; 49, 50, 525, 784, 800, 810 and 840 in FP64, where F^3 is up to 2.2 times (2n)^3).  Gains
 // at equal work: about 2 in FP64 (pipe-bound in both), 2.5 in double-float, 4 and more in FP32,
 // four times that where an axis needs Bluestein's algorithm (512x512x3, growth 2.7: FP64 0.53,
 // double-float 0.96, FP32 1.73 times the speed; 129^3: 11, 12 and 18 times).  Grids of up to

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__((N / PlanOf<ZKey<R>, N>::E) * rag_pairs_max<R,
 // Columns of a CTA of a line pass: 8 (128 bytes of a row at 16-byte values), 4 where a line
 // has 32 threads or more (smaller CTAs wait less at their barriers: double-float at 320 to
 // 768 4 to 12 % faster than 8; 2 loses more to half-used sectors), more where a line has
-// fewer than eight threads; halved while that leaves fewer than two CTAs an SM.
+// fewer than eight threads; halved while that leaves fewer than two CTAs on each of 152 SMs.
 template <class R, int N> int rag_tile(int T, int bmax, long long columns, long long outer)
 {
     int b = T >= 32 && sizeof(cpx<R>) >= 16 ? 4 : 8;
@@ -107,8 +107,10 @@ inline int rag_pairs(int T, int bmax, long long pairs)
 // 172 / 144), forward passes, whose loads are half as many, from 400 (200^3 47 / 41, 250^3
 // 102 / 72; 240x180x75 24.8 / 26.7).  Few tiles leave the persistent CTAs without a next one to
 // load (39x172x122, 1326 tiles, three a CTA: 3 % slower; 240x180x75, 2640: 2 % faster): from 16
-// an SM.  Eight values a thread have warps enough without it, and the x pass computes twice as
-// long a byte (200^3 117 / 144).
+// an SM (152 of them).  Eight values a thread have warps enough without it, and the x pass
+// computes twice as long a byte (200^3 117 / 144).  Above 864 all but the forward pass at 1280
+// need more than 110 KB; that one would gain (100x600x100 64 / 56, 200x640x100 131 / 101) and
+// is left on the plain tile.
 constexpr long long kPipeTiles = 16 * 152;
 template <class R, int N, int MODE> constexpr bool rag_pipe()
 {

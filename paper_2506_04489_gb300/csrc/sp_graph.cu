@@ -38,7 +38,7 @@ extern "C" sp_status sp_plan_autotune(sp_plan p, int batch, sp_stream stream)
         return sp_fail(SP_ERR_INVALID, "batch %d outside [1, max_batch = %d]", batch, p->max_batch);
     if (sp_status rc = sp_check_device(p)) return rc;
     for (int ax = 0; ax < 3; ++ax)
-        if (!sp_v2_supported(p->N[ax])) return SP_OK;  // first-generation passes: nothing to tune
+        if (!sp_v2_supported(p->N[ax])) return SP_OK;  // tiles by rule (sp_embed.cuh, sp_passes.cu): nothing to tune
     cudaStream_t st = (cudaStream_t)stream;
     const int candidates[6] = {1, 2, 4, 8, 16, 32};
     int best_tile[3] = {0, 0, 0}, best_variant[3] = {0, 0, 0};

@@ -3,9 +3,10 @@
 //   K5  1D integral tables G, H of eq. (Gten_sep) per axis
 //   K6  multiplier M_k = -|kappa|^2 Vhat_k / Ntilde (eqs. Gten_sep, convtheorem)
 //   K7  FFT twiddles exp(-2 pi i j / N)
-// K5 and K6 are both contractions over a long index (quadrature nodes, GS terms) and
-// run through one tiled FP64 GEMM kernel with problem-specific prologue/epilogue
-// kernels.
+//   and, for passes on lengths F > 2n, the multiplier of period F (sp_embed.cuh)
+// K5, K6 and the change of period are contractions over a long index (quadrature nodes, GS
+// terms, wavenumbers), each in a tiled FP64 kernel of its shape: k_axis_sums, k_dgemm_nt with
+// problem-specific operands and epilogues, k_dgemm_nn along strided axes.
 #include <math.h>
 #include <stdio.h>
 

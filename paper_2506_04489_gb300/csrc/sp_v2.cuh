@@ -321,8 +321,9 @@ SP_D void line_tile(const LArgs& a, int cb, int o, int batch, unsigned char* smr
         }
     }
     // x pass: the multiplier values of this thread's outputs are fetched before the forward
-    // transform, so their latency overlaps its arithmetic: into registers for FP32, into
-    // shared memory by cp.async for the 8-byte types (whose registers hold the transform)
+    // transform, so their latency overlaps its arithmetic: into registers for FP32 of fewer
+    // than 12 values a thread, into shared memory by cp.async for the rest (whose registers
+    // hold the transform)
     constexpr bool ROW_M = row_m<R, N, MODE, K>();
     constexpr bool PREFETCH_M = MODE == XMUL && sizeof(R) == 4 && !ROW_M;
     constexpr bool STAGE_M = stage_m<R, MODE>();
